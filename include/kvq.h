@@ -456,8 +456,9 @@ int32_t kvq_drift_max_vocab(void);
  *              each row (vocab a multiple of 4) gives vector loads.
  *   m_t        device int32 [rows]; c_t, d_loc device fp32 [rows];
  *   y_t        device uint8 [rows]; cov device fp32 [rows][k_max].
- * Probabilities are e^(z - max z) in fp32, summed in fp64 (c_t, d_loc are
- * the fp64 results rounded to fp32).  rows <= 65535, vocab <= 163840.
+ * Probabilities are e^(z - max z) in fp32; masses are summed as multiples of
+ * 2^-40, products in double-float, and combined in fp64 (c_t, d_loc are the
+ * fp64 results rounded to fp32).  rows <= 65535, vocab <= 163840.
  * No workspace; calls on different outputs may overlap.
  */
 kvq_status kvq_drift_metrics(const float* z_fp, const float* z_q, int32_t rows,
@@ -469,7 +470,9 @@ kvq_status kvq_drift_metrics(const float* z_fp, const float* z_q, int32_t rows,
  * kvq_drift_window — K_b of Sec. 4.1: the smallest k whose coverage
  * cov[.][k-1], averaged over the rows, reaches rho_k; 0 if none does.
  *   cov       device fp32 [rows][k_max] (from kvq_drift_metrics).
- *   mean_cov  device fp32 [k_max]: the column means (fp64 sums, row order).
+ *   mean_cov  device fp32 [k_max]: the column means (compensated fp32 sums of
+ *             each thread's rows, good to 2^-46, added in fp64 in a fixed
+ *             order).
  *   k_b       device int32 [1].
  */
 kvq_status kvq_drift_window(const float* cov, int32_t rows, int32_t k_max,

@@ -543,8 +543,8 @@ kvq_status kvq_drift_metrics(const float* z_fp, const float* z_q, int32_t rows, 
     return fail(KVQ_ERR_ARG, "window must be in [1, k_max] (got %d)", p->window);
   if (!isfinite(p->eps) || !isfinite(p->rho_c))
     return fail(KVQ_ERR_ARG, "eps and rho_c must be finite");
-  trace("kvq_drift_metrics rows %d vocab %d alpha %g window %d k_max %d grid (8, %d) x 512, "
-        "clusters of 8", rows, vocab, (double)p->alpha, p->window, p->k_max, rows);
+  trace("kvq_drift_metrics rows %d vocab %d alpha %g window %d k_max %d grid (%d)", rows,
+        vocab, (double)p->alpha, p->window, p->k_max, rows);
   return cuda_status(launch_drift(z_fp, z_q, rows, vocab, *p, m_t, c_t, d_loc, y_t, cov,
                                   static_cast<cudaStream_t>(stream)),
                      "kvq_drift_metrics launch");

@@ -14,9 +14,15 @@
 //   cov_t(k)  sum of p_fp over C and TopK(z_q, k), k = 1 .. k_max.
 // K_b is the smallest k whose coverage averaged over the rows reaches rho_K.
 //
-// One cluster of 8 CTAs per row.  Each CTA stages an eighth of both logit
-// rows in shared memory once (the only HBM read) and the CTAs combine their
-// partial results through distributed shared memory:
+// Two kernels.  The streaming kernel (below) takes every row with one CTA; a
+// row that its guesses do not settle (thousands of nearly equal logits around
+// a boundary, alpha = 1) it leaves to the general kernel, launched behind it,
+// which takes any row with one cluster of 8 CTAs.  256 rows of 128256 on a
+// GB300: 1050 us with the general kernel alone, 160 with both.
+//
+// The general kernel.  Each CTA stages an eighth of both logit rows in shared
+// memory once (the only HBM read) and the CTAs combine their partial results
+// through distributed shared memory:
 //   1. maxima;
 //   2. the FP16 boundary: a 2048-bin histogram of the depth (m - z) * 64
 //      (count and mass per bin, the depth order is the FP16 order) and, in
@@ -186,6 +192,12 @@ __device__ __forceinline__ uint32_t pk_idx(unsigned long long w) {
   return 0xffffffffu - (uint32_t)w;
 }
 
+// Programmatic dependent launch (no-ops without the launch attribute).
+__device__ __forceinline__ void pdl_launch_dependents() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ---- block reductions (all threads get the result) ----
 __device__ u64 block_sum_q(u64 v, Sm& s) {
 #pragma unroll
@@ -195,27 +207,6 @@ __device__ u64 block_sum_q(u64 v, Sm& s) {
   __syncthreads();
   u64 r = 0ull;
   for (int w = 0; w < kW; ++w) r += s.rq[w];
-  return r;
-}
-__device__ Df block_sum_df(Df v, Sm& s) {
-#pragma unroll
-  for (int o = 16; o; o >>= 1) {
-    Df w;
-    w.hi = __shfl_xor_sync(0xffffffffu, v.hi, o);
-    w.lo = __shfl_xor_sync(0xffffffffu, v.lo, o);
-    // a fixed pairing order keeps every lane's result identical
-    if ((threadIdx.x & o) == 0) {
-      v.add(w);
-    } else {
-      w.add(v);
-      v = w;
-    }
-  }
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) s.rq[threadIdx.x >> 5] = v.pack();
-  __syncthreads();
-  Df r;
-  for (int w = 0; w < kW; ++w) r.add(Df::unpack(s.rq[w]));
   return r;
 }
 __device__ float block_max_f(float v, Sm& s) {
@@ -320,27 +311,34 @@ __device__ void cluster_red2_u(Sm& s, int slot, uint32_t& a, uint32_t& b, int op
   b = rb;
 }
 
-// Bitonic sort of buf[0, n) descending (n <= kCap), padding with 0.
-__device__ void sort_desc(Sm& s, int n) {
+// Bitonic sort of buf[0, n) descending (n <= kCap), padding with 0.  A step
+// of distance j <= 16 stays inside the 32 consecutive elements that one warp
+// handles, so only the longer steps need the block's barrier.
+template <int kN>
+__device__ void sort_desc(u64* buf, int n) {
   int P = 2;
   while (P < n) P <<= 1;
-  for (int i = n + threadIdx.x; i < P; i += kT) s.buf[i] = 0ull;
+  __syncthreads();
+  for (int i = n + threadIdx.x; i < P; i += kN) buf[i] = 0ull;
   __syncthreads();
   for (int k = 2; k <= P; k <<= 1)
     for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int i = threadIdx.x; i < P; i += kT) {
+      for (int i = threadIdx.x; i < P; i += kN) {
         const int ixj = i ^ j;
         if (ixj > i) {
-          const unsigned long long a = s.buf[i], b = s.buf[ixj];
+          const unsigned long long a = buf[i], b = buf[ixj];
           const bool desc = (i & k) == 0;
           if (desc ? (a < b) : (a > b)) {
-            s.buf[i] = b;
-            s.buf[ixj] = a;
+            buf[i] = b;
+            buf[ixj] = a;
           }
         }
       }
-      __syncthreads();
+      const int next = j > 1 ? j >> 1 : k;  // the next step's distance
+      if (j > 16 || next > 16) __syncthreads();
+      else __syncwarp();
     }
+  __syncthreads();
 }
 
 struct Ctx {
@@ -708,7 +706,7 @@ __device__ Pick select(Sm& s, const Ctx& cx, const float* a, float m, bool weigh
   cluster_sync();
   if (cx.rank == 0) {
     const int n = (int)min(s.nbuf, (uint32_t)kCap);
-    sort_desc(s, n);
+    sort_desc<kT>(s.buf, n);
     if (threadIdx.x < 32) {
       // first element whose prefix weight (above + own) reaches the target
       const int l = threadIdx.x;
@@ -751,13 +749,45 @@ __device__ __forceinline__ bool ranks_in(uint32_t k, uint32_t i, const Pick& p) 
   return p.all || k > p.key || (k == p.key && i <= p.idx);
 }
 
-__global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kT, 1)
-    drift_kernel(const float* __restrict__ z_fp, const float* __restrict__ z_q, int vocab,
-                 kvq_drift_params p, int32_t* __restrict__ m_t, float* __restrict__ c_t,
-                 float* __restrict__ d_loc, uint8_t* __restrict__ y_t, float* __restrict__ cov) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  Sm& s = *reinterpret_cast<Sm*>(smem_raw);
-  const int row = blockIdx.y;
+// Row results from the masses A = e_fp(U), B = e_q(U), c_sum = e_fp(C and S),
+// S_fp and the product sums (one thread).
+__device__ void write_row(int row, int32_t len, u64 A, u64 B, u64 c_sum, double sf, const Df& saa,
+                          const Df& sab, const Df& sbb, const kvq_drift_params& p, int32_t* m_t,
+                          float* c_t, float* d_loc, uint8_t* y_t) {
+  const double ia = kFix / (double)A, ib = kFix / (double)B;
+  double dsum = saa.value() * ia * ia - 2.0 * sab.value() * ia * ib + sbb.value() * ib * ib;
+  if (dsum < 0.0) dsum = 0.0;  // rounding of an exact zero
+  const double c = (double)c_sum / sf;
+  const double d = sqrt(dsum);
+  m_t[row] = len;
+  c_t[row] = (float)c;
+  d_loc[row] = (float)d;
+  y_t[row] = (uint8_t)(d > (double)p.eps && c >= (double)p.rho_c);
+}
+// The coverage curve: prefix sums of the terms wsel over S_fp (one warp).
+__device__ void write_curve(const u64* wsel, double sf, int row, int k_max, float* cov) {
+  const int l = threadIdx.x & 31;
+  const float inv = (float)(1.0 / sf);
+  u64 run = 0ull;
+  for (int j0 = 0; j0 < k_max; j0 += 32) {
+    const int j = j0 + l;
+    u64 inc = j < k_max ? wsel[j] : 0ull;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const u64 t = __shfl_up_sync(0xffffffffu, inc, o);
+      if (l >= o) inc += t;
+    }
+    if (j < k_max) cov[(long long)row * k_max + j] = (float)(run + inc) * inv;
+    run += __shfl_sync(0xffffffffu, inc, 31);
+  }
+}
+
+// One row of the general kernel (the CTAs of one cluster).
+__device__ void drift_row(Sm& s, const float* __restrict__ z_fp, const float* __restrict__ z_q,
+                          int row, int vocab, const kvq_drift_params& p,
+                          int32_t* __restrict__ m_t, float* __restrict__ c_t,
+                          float* __restrict__ d_loc, uint8_t* __restrict__ y_t,
+                          float* __restrict__ cov) {
   Ctx cx;
   cx.rank = cluster_rank();
   const int sl = ((vocab + kCl - 1) / kCl + 3) & ~3;
@@ -817,7 +847,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kT, 1)
       [&](int i) { return fkey(s.zq[i]); });
   cluster_sync();
   if (cx.rank == 0) {
-    sort_desc(s, (int)min(s.nbuf, (uint32_t)kCap));
+    sort_desc<kT>(s.buf, (int)min(s.nbuf, (uint32_t)kCap));
     if (threadIdx.x == 0) {
       const unsigned long long w = s.buf[p.window - 1];  // the K-th of TopK(z_q)
       s.res_u[4] = pk_key(w);
@@ -934,33 +964,24 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kT, 1)
   cluster_gather2x(s, slot, A, B, Cs, saa.pack(), sab.pack(), sbb.pack());
   slot += 2;
   u64 c_sum = 0ull;
-  double Dsum = 0.0;
   if (threadIdx.x == 0) {
     A = B = 0ull;
-    Df taa, tab, tbb;
+    saa = sab = sbb = Df();
     for (int r = 0; r < kCl; ++r) {
       A += s.xin8[r][0];
       B += s.xin8[r][1];
       c_sum += s.xin8[r][2];
-      taa.add(Df::unpack(s.xin8[r][3]));
-      tab.add(Df::unpack(s.xin8[r][4]));
-      tbb.add(Df::unpack(s.xin8[r][5]));
+      saa.add(Df::unpack(s.xin8[r][3]));
+      sab.add(Df::unpack(s.xin8[r][4]));
+      sbb.add(Df::unpack(s.xin8[r][5]));
     }
-    const double ia = kFix / (double)A, ib = kFix / (double)B;
-    Dsum = taa.value() * ia * ia - 2.0 * tab.value() * ia * ib + tbb.value() * ib * ib;
-    if (Dsum < 0.0) Dsum = 0.0;  // rounding of an exact zero
   }
 
   // ---- outputs (rank 0) ----
   if (cx.rank == 0) {
-    if (threadIdx.x == 0) {
-      const double c = (double)c_sum / (double)sf;
-      const double d = sqrt(Dsum);
-      m_t[row] = pf.all ? vocab : (int32_t)pf.len;
-      c_t[row] = (float)c;
-      d_loc[row] = (float)d;
-      y_t[row] = (uint8_t)(d > (double)p.eps && c >= (double)p.rho_c);
-    }
+    if (threadIdx.x == 0)
+      write_row(row, pf.all ? vocab : (int32_t)pf.len, A, B, c_sum, (double)sf, saa, sab,
+                sbb, p, m_t, c_t, d_loc, y_t);
     // coverage curve: prefix sums of p_fp over TopK(z_q, k) within C; the
     // FP16 logits of the list come from the CTAs that hold them
     const int sl = ((vocab + kCl - 1) / kCl + 3) & ~3;
@@ -974,50 +995,866 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kT, 1)
       }
       s.wsel[threadIdx.x] = w;
     }
-    if (threadIdx.x == 0) s.bc[2] = (float)(1.0 / (double)sf);
     __syncthreads();
-    if (threadIdx.x < 32) {
-      const int l = threadIdx.x;
-      const float inv = s.bc[2];
-      u64 run = 0ull;
-      for (int j0 = 0; j0 < p.k_max; j0 += 32) {
-        const int j = j0 + l;
-        u64 inc = j < p.k_max ? s.wsel[j] : 0ull;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const u64 t = __shfl_up_sync(0xffffffffu, inc, o);
-          if (l >= o) inc += t;
-        }
-        if (j < p.k_max) cov[(long long)row * p.k_max + j] = (float)(run + inc) * inv;
-        run += __shfl_sync(0xffffffffu, inc, 31);
-      }
-    }
+    if (threadIdx.x < 32) write_curve(s.wsel, (double)sf, row, p.k_max, cov);
   }
-  cluster_sync();  // no CTA leaves while a peer may read its shared memory
+  cluster_sync();  // no CTA goes on while a peer may read its shared memory
 }
 
-// K_b: column means of cov over the rows (fixed order, fp64) and the smallest
-// k whose mean reaches rho_K (0 if none).
-__global__ void __launch_bounds__(256) drift_window_kernel(const float* __restrict__ cov, int rows,
-                                                           int k_max, float rho_k,
-                                                           float* __restrict__ mean_cov,
-                                                           int32_t* __restrict__ k_b) {
-  __shared__ int best[8];
-  int mine = 0x7fffffff;
-  for (int k = threadIdx.x; k < k_max; k += blockDim.x) {
-    double sum = 0.0;
-    for (int r = 0; r < rows; ++r) sum += (double)cov[(long long)r * k_max + k];
-    const double mean = sum / rows;
-    mean_cov[k] = (float)mean;
-    if (mean >= (double)rho_k) mine = min(mine, k + 1);
+__global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kT, 1)
+    drift_general_kernel(const float* __restrict__ z_fp, const float* __restrict__ z_q, int rows,
+                         int vocab, kvq_drift_params p, int32_t* __restrict__ m_t,
+                         float* __restrict__ c_t, float* __restrict__ d_loc,
+                         uint8_t* __restrict__ y_t, float* __restrict__ cov) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  Sm& s = *reinterpret_cast<Sm*>(smem_raw);
+  pdl_launch_dependents();
+  pdl_wait();  // the streaming kernel's marks
+  // Marks are read kT rows at a time (usually none is set).  Every CTA of the
+  // cluster reads them before the barriers that come before rank 0 overwrites
+  // one.
+  for (int r0 = blockIdx.y; r0 < rows; r0 += kT * (int)gridDim.y) {
+    const int mine = r0 + (int)threadIdx.x * (int)gridDim.y;
+    const bool left = mine < rows && *reinterpret_cast<volatile int32_t*>(m_t + mine) < 0;
+    if (!__syncthreads_or(left)) continue;
+    const uint32_t bal = __ballot_sync(0xffffffffu, left);
+    __shared__ uint32_t marks[kT / 32];
+    if ((threadIdx.x & 31) == 0) marks[threadIdx.x >> 5] = bal;
+    __syncthreads();
+    for (int k = 0; k < kT; ++k)
+      if (marks[k >> 5] >> (k & 31) & 1u)
+        drift_row(s, z_fp, z_q, r0 + k * (int)gridDim.y, vocab, p, m_t, c_t, d_loc, y_t, cov);
+    __syncthreads();
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The streaming kernel: one CTA per row, the logits read straight from global
+// memory; 512 threads, two rows per SM, or 1024 threads for launches of at
+// most one row per SM.
+//
+//   sample  eight runs of elements spread over the row: where the histogram's
+//           grid begins, and below which logits neither boundary can lie.
+//   pass A  both rows once (the HBM read): maxima, a guess of S_fp (relative
+//           to the sample's maximum), a count per 1/64 unit of z_fp logit
+//           (shared-memory histogram) and the positions of the z_q logits
+//           above the sample's bound.
+//   plan    a few bins around the place where the prefix mass should reach
+//           alpha (each bin weighed by the exponential of its centre), and
+//           the bin where the count of z_q reaches k_max.
+//   pass B  z_fp again (from L2 as far as it holds it): S_fp; elements above
+//           the bins (certainly in C) add to the masses and the d_loc sums;
+//           the few hundred inside the bins are listed.  The noted z_q logits
+//           down to its bin are listed too.
+//   finish  the exact boundary element among the listed ones (the masses
+//           above them must bracket the target, which is checked), the z_q
+//           list sorted, the listed members of U added, the row written.
+//
+// The sample, the guess of S_fp and the histogram only steer: masses,
+// comparisons and orders are the ones defined above, over the same exact
+// integers as in the general kernel, so a bad guess is noticed.  A row that is
+// not settled (more than kL nearly equal logits at a boundary, a boundary more
+// than 20 units below the sample's maximum, a sample far from the row) is
+// marked m_t = -1 and left to the general kernel, launched behind it.
+//
+// What bounds it: the HBM reads (both rows, and z_fp once more beyond what L2
+// keeps), then the latency of the serial steps of a row; one CTA per row has
+// block barriers only and keeps up to 304 rows in flight, where a cluster of
+// 2, 4 or 8 CTAs per row spent 25 us per row on cluster barriers and
+// distributed shared memory (190, 203 and 230 us for 256 rows of 128256).
+// ---------------------------------------------------------------------------
+
+constexpr int kL = 1024;             // listed elements of a row
+constexpr int kUp = 12;              // units above the sample's maximum in the histogram
+constexpr uint32_t kSpread = 300;    // elements listed on either side of the estimate
+constexpr float kMagic = 8388608.0f; // 2^23: floats in [2^23, 2^24) are whole numbers
+constexpr int kU = 2;                // 16-byte loads of the next step in flight per thread
+constexpr int kRuns = 8;             // sample elements per thread
+constexpr int kMemCap = 16;          // members a thread notes before its warp works on them
+constexpr int kTopCap = 12;          // z_q candidates a thread notes
+
+template <int kS>
+struct Ss {
+  static constexpr int kSw = kS / 32;
+  union {
+    uint32_t hf[kBins];           // pass A
+    u64 lf[kL];                   // pass B: z_fp elements inside the bins
+  };
+  union {
+    uint32_t hq[kBins];           // z_q counts
+    uint16_t mem[kMemCap][kS];    // pass B: positions of members
+    u64 mass[kL];                 // finish: masses of the listed elements' key ranges
+  };
+  u64 lq[kL];                     // pass B: z_q elements down to the k_max bin
+  u64 top[kL];                    // the same, best first
+  uint16_t cand[kTopCap][kS];     // pass A: positions of z_q candidates
+  union {
+    uint16_t flat[kSw][32 * kMemCap];  // a warp's members, side by side
+    u64 set[kS];                  // finish: the elements around the boundary
+  };
+  u64 wsel[kMaxKcov];             // coverage terms
+  u64 part[kSw][8];               // warps' sums: count, A, B, C and S, saa, sab, sbb
+  u64 su[kSw], sv[kSw];
+  float rf[3][kSw];
+  uint32_t sc[2][kSw];
+  uint32_t pick[12];
+  uint32_t nf, nq;                // list lengths
+};
+
+// A row of n floats (4-byte aligned) as each thread streams it: vectors
+// u = 0, 1, ... of thread t at 16-byte positions u kS + t past the first
+// boundary, then one vector with the single elements before and after them
+// (missing elements are -inf).
+template <int kS>
+struct Stream {
+  const float* p;
+  int head, nv, n, steps;  // steps: full vectors per thread (the last may be empty)
+  __device__ Stream(const float* q, int m) : p(q), n(m) {
+    head = min(m, (int)((16u - (reinterpret_cast<uintptr_t>(q) & 15u)) & 15u) >> 2);
+    nv = (m - head) >> 2;
+    steps = (nv + kS - 1) / kS;
+  }
+  // Index of element k of vector u of thread t.
+  __device__ __forceinline__ int index(int t, int u, int k) const {
+    return u < steps ? head + 4 * (u * kS + t) + k : (t < head ? t : 4 * nv + t);
+  }
+  __device__ __forceinline__ float4 load(int u) const {
+    const int j = u * kS + (int)threadIdx.x;
+    return j < nv ? __ldg(reinterpret_cast<const float4*>(p + head) + j)
+                  : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+  }
+  // f(vector, u) for every vector of this thread; all threads call f equally
+  // often.  The next kU loads are issued before the current ones are used.
+  template <typename F>
+  __device__ __forceinline__ void each(const F& f) const {
+    float4 v[kU], w[kU];
+#pragma unroll
+    for (int k = 0; k < kU; ++k) v[k] = load(k);
+    for (int u = 0; u < steps; u += kU) {
+#pragma unroll
+      for (int k = 0; k < kU; ++k) w[k] = load(u + kU + k);
+#pragma unroll
+      for (int k = 0; k < kU; ++k)
+        if (u + k < steps) f(v[k], u + k);
+#pragma unroll
+      for (int k = 0; k < kU; ++k) v[k] = w[k];
+    }
+    const int ends = n - 4 * nv;
+    if (ends > 0) {
+      float4 e = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+      if ((int)threadIdx.x < ends) e.x = p[index(threadIdx.x, steps, 0)];
+      f(e, steps);
+    }
+  }
+};
+// positions (vector, lane, element) fit 16 bits
+static_assert((kCl * kSlice / 4 / 512 + 2) * 128 <= 65536, "positions fit 16 bits");
+
+__device__ __forceinline__ float max4(const float4& v) {
+  return fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w));
+}
+// About e^(z - m), for the plan only.
+__device__ __forceinline__ float exp_guess(float z, float m) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(fmaf(z, 1.44269504f, -1.44269504f * m)));
+  return y;
+}
+// The integer a (even) whose bin a - 64 z is 0 for z = kUp units above x.
+__device__ __forceinline__ int bin_origin(float x) {
+  const float a = 2.0f * rintf((kDepthScale / 2.0f) * (x + (float)kUp));
+  return fabsf(a) < 4194304.0f ? (int)a : 0;  // |a| < 2^22 (and not NaN), else the guess is void
+}
+// The bin of z on the grid of origin a, clamped at bin 0 (z >= bin_floor(a)),
+// as a float 2^23 + bin; without the clamp it orders all z alike.
+__device__ __forceinline__ float bin_place(float z, float a) {
+  return fmaf(-kDepthScale, z, a + kMagic);
+}
+__device__ __forceinline__ uint32_t bin_of(float z, float a) {
+  return __float_as_uint(fmaxf(bin_place(z, a), kMagic)) - 0x4b000000u;
+}
+__device__ __forceinline__ float bin_floor(float a) {
+  return (a - (float)(kBins - 1)) * (1.0f / kDepthScale);
+}
+
+// Compensated sum: hi + lo, lo collecting the rounding errors of hi.
+struct Cs {
+  float hi = 0.0f, lo = 0.0f;
+  __device__ __forceinline__ void add(float x, float rest = 0.0f) {
+    const float s = hi + x;
+    const float b = s - hi;
+    lo += ((hi - (s - b)) + (x - b)) + rest;
+    hi = s;
+  }
+  __device__ __forceinline__ void add_prod(float a, float b) {
+    const float p = a * b;
+    add(p, fmaf(a, b, -p));
+  }
+  __device__ __forceinline__ Df df() const {
+    Df d;
+    d.add(hi);
+    d.add(lo);
+    return d;
+  }
+};
+// A sum of terms e in [0, 1] as multiples of 2^-40 (fix40's value, at most
+// 4095 terms): e + 8 rounds e to a multiple of 2^-20, the exact rest + 1.5
+// 2^-17 to one of 2^-40.
+struct Fixed {
+  uint32_t hi = 0u, lo = 0u;
+  __device__ __forceinline__ void add(float e) {
+    const float h = e + 8.0f;
+    hi += __float_as_uint(h) - 0x41000000u;
+    lo += __float_as_uint((e - (h - 8.0f)) + 1.5f / 131072.0f) - 0x37400000u;
+  }
+  __device__ __forceinline__ u64 value() const {
+    return ((u64)hi << 20) + (u64)(long long)(int)lo;
+  }
+};
+// A thread's sums over members of U.
+struct Sums {
+  uint32_t cnt = 0u;
+  Fixed A, B;
+  u64 C = 0ull;
+  Cs aa, ab, bb;
+  __device__ __forceinline__ void add(float a, float b) {
+    A.add(a);
+    B.add(b);
+    aa.add_prod(a, a);
+    ab.add_prod(a, b);
+    bb.add_prod(b, b);
+  }
+};
+__device__ __forceinline__ void df_xor(Df& v, int o) {  // a fixed pairing order
+  Df w;
+  w.hi = __shfl_xor_sync(0xffffffffu, v.hi, o);
+  w.lo = __shfl_xor_sync(0xffffffffu, v.lo, o);
+  const bool up = (threadIdx.x & o) != 0;
+  const Df a = up ? w : v, b = up ? v : w;
+  v = a;
+  v.add(b);
+}
+// Sums over the warp into words out[0..6], by lane 0.
+__device__ __forceinline__ void warp_sums(u64 n, u64 A, u64 B, u64 C, Df aa, Df ab, Df bb,
+                                          u64* out) {
+#pragma unroll
+  for (int o = 16; o; o >>= 1) {
+    n += __shfl_xor_sync(0xffffffffu, n, o);
+    A += __shfl_xor_sync(0xffffffffu, A, o);
+    B += __shfl_xor_sync(0xffffffffu, B, o);
+    C += __shfl_xor_sync(0xffffffffu, C, o);
+    df_xor(aa, o);
+    df_xor(ab, o);
+    df_xor(bb, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    out[0] = n;
+    out[1] = A;
+    out[2] = B;
+    out[3] = C;
+    out[4] = aa.pack();
+    out[5] = ab.pack();
+    out[6] = bb.pack();
+  }
+}
+__device__ __forceinline__ void warp_sums(const Sums& v, u64* out) {
+  warp_sums(v.cnt, v.A.value(), v.B.value(), v.C, v.aa.df(), v.ab.df(), v.bb.df(), out);
+}
+
+// Exclusive prefix of x over the threads; *total the sum.  buf: one word per
+// warp, not read by anyone when the call begins.
+template <int kS, typename T>
+__device__ __forceinline__ T scan(T x, T* buf, T* total) {
+  const int l = threadIdx.x & 31, w = threadIdx.x >> 5;
+  T i = x;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const T y = __shfl_up_sync(0xffffffffu, i, o);
+    if (l >= o) i += y;
+  }
+  if (l == 31) buf[w] = i;
+  __syncthreads();
+  T before = 0, all = 0;
+#pragma unroll
+  for (int v = 0; v < kS / 32; ++v) {
+    const T y = buf[v];
+    before += v < w ? y : (T)0;
+    all += y;
+  }
+  *total = all;
+  return before + i - x;
+}
+
+// The bins [b1, b2] of z_fp to list, around the place where the prefix mass
+// should reach `goal` (in units of e^top), into pick[3..4] (pick[7] = 1 if they hold at most kL
+// elements), and the bin of z_q where the count reaches k_max into pick[8]
+// (pick[9] = 1 if at most kL elements rank above or in it).
+template <int kS>
+__device__ void make_plan(Ss<kS>& s, float top, float a_f, float goal, uint32_t k_max) {
+  constexpr int kPer = kBins / kS;
+  const int t = threadIdx.x;
+  if (t < 12) s.pick[t] = t == 0 || t == 8 ? kBins : 0u;
+  uint32_t c[kPer], cs = 0u, d[kPer], ds = 0u;
+  float w[kPer], ws = 0.0f;
+  const float b0 = fmaf(-kDepthScale, top, a_f);  // its place among the bins (maybe below 0)
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    c[k] = s.hf[kPer * t + k];
+    d[k] = s.hq[kPer * t + k];
+    // bin 0 may hold elements above it: weighed like the maximum
+    const float b = kPer * t + k == 0 ? fminf(b0, 0.0f) : (float)(kPer * t + k);
+    w[k] = (float)c[k] * exp2f((b0 - b) * (1.44269504f / kDepthScale));
+    cs += c[k];
+    ds += d[k];
+    ws += w[k];
+  }
+  float all_w;
+  uint32_t all_c, all_d;
+  const float wb = scan<kS>(ws, s.rf[0], &all_w);
+  uint32_t x = scan<kS>(cs, s.sc[0], &all_c), y = scan<kS>(ds, s.sc[1], &all_d);
+  {
+    uint32_t b = kBins;  // the first bin whose prefix mass reaches the goal
+    float q = wb;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      q += w[k];
+      if (b == (uint32_t)kBins && c[k] > 0u && q >= goal) b = (uint32_t)(kPer * t + k);
+      if (y < k_max && y + d[k] >= k_max) {
+        s.pick[8] = (uint32_t)(kPer * t + k);
+        s.pick[9] = y + d[k] <= (uint32_t)kL ? 1u : 0u;
+      }
+      y += d[k];
+    }
+    if (b < (uint32_t)kBins) atomicMin(&s.pick[0], b);
+  }
+  __syncthreads();
+  const uint32_t bc = s.pick[0];
+  if (bc / kPer == (uint32_t)t) {  // counts before it and up to it
+    uint32_t u = x, v = 0u;
+#pragma unroll
+    for (uint32_t k = 0; k < (uint32_t)kPer; ++k) {
+      u += k < bc % kPer ? c[k] : 0u;
+      v = k == bc % kPer ? c[k] : v;
+    }
+    s.pick[1] = u;
+    s.pick[2] = u + v;
+    s.pick[3] = bc;
+    s.pick[4] = bc;
+  }
+  __syncthreads();
+  if (bc < (uint32_t)kBins) {
+    const uint32_t c0 = s.pick[1], c1 = s.pick[2];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const uint32_t b = (uint32_t)(kPer * t + k);
+      if (b < bc && x + c[k] + kSpread > c0) atomicMin(&s.pick[3], b);
+      if (b > bc && x < c1 + kSpread) atomicMax(&s.pick[4], b);
+      x += c[k];
+    }
+  }
+  __syncthreads();
+  {
+    const uint32_t b1 = s.pick[3], b2 = s.pick[4];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {  // the elements in them
+      const uint32_t b = (uint32_t)(kPer * t + k);
+      if (b >= b1 && b <= b2 && c[k]) atomicAdd(&s.pick[5], c[k]);
+    }
+  }
+  __syncthreads();
+  if (t == 0) {
+    const bool wide = s.pick[5] <= (uint32_t)kL;
+    if (!wide) s.pick[3] = s.pick[4] = bc;
+    s.pick[7] = bc < (uint32_t)kBins && (wide || s.pick[2] - s.pick[1] <= (uint32_t)kL) ? 1u : 0u;
+  }
+  __syncthreads();
+}
+
+// The first of the n listed z_fp elements, in order, whose prefix mass (on
+// top of `above`) reaches `target`, into pick[0..1] (key, index), with
+// pick[2] = 1.  The elements' key range is cut into kL parts, the part where
+// the mass reaches the target is found by a scan, and the few elements in it
+// are compared pairwise (pick[2] = 0 if they are more than kS, or the target
+// lies elsewhere).
+template <int kS>
+__device__ void find_boundary(Ss<kS>& s, int n, u64 above, u64 target, float mf) {
+  constexpr int kPer = kL / kS;
+  const int t = threadIdx.x, l = t & 31, w = t >> 5;
+  uint32_t lo = 0xffffffffu, hi = 0u;
+  for (int j = t; j < n; j += kS) {
+    const uint32_t k = pk_key(s.lf[j]);
+    lo = min(lo, k);
+    hi = max(hi, k);
   }
 #pragma unroll
-  for (int o = 16; o; o >>= 1) mine = min(mine, __shfl_xor_sync(0xffffffffu, mine, o));
-  if ((threadIdx.x & 31) == 0) best[threadIdx.x >> 5] = mine;
+  for (int k = 0; k < kPer; ++k) s.mass[k * kS + t] = 0ull;
+  lo = __reduce_min_sync(0xffffffffu, lo);
+  hi = __reduce_max_sync(0xffffffffu, hi);
+  if (t == 0) {
+    s.pick[1] = s.pick[2] = s.pick[3] = 0u;
+    s.pick[0] = 0xffffffffu;
+    s.pick[4] = kL;
+  }
+  if (l == 0) {
+    s.sc[0][w] = lo;
+    s.sc[1][w] = hi;
+  }
   __syncthreads();
-  if (threadIdx.x == 0) {
+#pragma unroll
+  for (int v = 0; v < kS / 32; ++v) {
+    lo = min(lo, s.sc[0][v]);
+    hi = max(hi, s.sc[1][v]);
+  }
+  const int sh = n > 0 ? max(0, 22 - __clz(hi - lo)) : 0;  // (hi - lo) >> sh < 1024 = kL
+  auto part_of = [&](u64 e) { return (hi - pk_key(e)) >> sh; };
+  auto mass_of = [&](u64 e) { return fix40(expf(fval(pk_key(e)) - mf)); };
+  for (int j = t; j < n; j += kS) atomicAdd(&s.mass[part_of(s.lf[j])], mass_of(s.lf[j]));
+  __syncthreads();
+  u64 m[kPer], sum = 0ull, all;
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    m[k] = s.mass[kPer * t + k];
+    sum += m[k];
+  }
+  u64 run = above + scan<kS>(sum, s.su, &all);
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    if (run < target && target <= run + m[k]) {
+      s.pick[4] = (uint32_t)(kPer * t + k);
+      s.sv[0] = run;
+    }
+    run += m[k];
+  }
+  __syncthreads();
+  const uint32_t part = s.pick[4];
+  if (part >= (uint32_t)kL) return;
+  for (int j = t; j < n; j += kS) {
+    const u64 e = s.lf[j];
+    if (part_of(e) == part) {
+      const uint32_t q = atomicAdd(&s.pick[3], 1u);
+      if (q < (uint32_t)kS) s.set[q] = e;
+    }
+  }
+  __syncthreads();
+  const int k = (int)s.pick[3];
+  if (k <= kS && t < k) {
+    const u64 e = s.set[t], own = mass_of(e);
+    u64 pre = s.sv[0];
+    for (int j = 0; j < k; ++j)
+      if (s.set[j] > e) pre += mass_of(s.set[j]);
+    if (pre < target && target <= pre + own) {
+      s.pick[0] = pk_key(e);
+      s.pick[1] = pk_idx(e);
+      s.pick[2] = 1u;
+    }
+  }
+  __syncthreads();
+}
+
+template <int kS>
+__global__ void __launch_bounds__(kS, 1024 / kS)
+    drift_stream_kernel(const float* __restrict__ z_fp, const float* __restrict__ z_q, int vocab,
+                        kvq_drift_params p, int32_t* __restrict__ m_t, float* __restrict__ c_t,
+                        float* __restrict__ d_loc, uint8_t* __restrict__ y_t,
+                        float* __restrict__ cov) {
+  constexpr int kSw = kS / 32;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  Ss<kS>& s = *reinterpret_cast<Ss<kS>*>(smem_raw);
+  const int row = blockIdx.x, t = threadIdx.x, warp = t >> 5, lane = t & 31, n = vocab;
+  pdl_launch_dependents();
+  const float* rf = z_fp + (long long)row * vocab;
+  const float* rq = z_q + (long long)row * vocab;
+  const Stream<kS> f(rf, n), q(rq, n);
+
+  // ---- sample ----
+  // The grid begins kUp units above the sample's maximum (elements above go
+  // to bin 0, elements kBins / 64 units below are not counted).  z_fp below
+  // cut_f is not counted: with the smallest of four quarter-sample means of
+  // e^z as a low guess of the row's, all of it weighs less than half of the
+  // mass outside C.  z_q below cut_q, the least of the warps' maxima of 256
+  // elements (the upper 1.2% or 1.5% of the row in the middle), is not a
+  // candidate when k_max is under 1/400 of the vocabulary.
+  float mf = -INFINITY, mq = -INFINITY, cut_f, cut_q;
+  {
+    float z[kRuns];
+#pragma unroll
+    for (int u = 0; u < kRuns; ++u) {
+      const int i = n >= kRuns * kS ? u * (n / kRuns) + t : u * kS + t;
+      z[u] = i < n ? __ldg(rf + i) : -INFINITY;
+      mf = fmaxf(mf, z[u]);
+      mq = fmaxf(mq, i < n ? __ldg(rq + i) : -INFINITY);
+    }
+    for (int i = t; i < kBins; i += kS) s.hf[i] = s.hq[i] = 0u;
+    if (t == 0) s.nf = s.nq = 0u;
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+      mf = fmaxf(mf, __shfl_xor_sync(0xffffffffu, mf, o));
+      mq = fmaxf(mq, __shfl_xor_sync(0xffffffffu, mq, o));
+    }
+    // (a warp's terms are relative to its own maximum)
+    float e = 0.0f;
+#pragma unroll
+    for (int u = 0; u < kRuns; ++u)
+      e += z[u] > -INFINITY ? exp2f((z[u] - mf) * 1.44269504f) : 0.0f;
+#pragma unroll
+    for (int o = 16; o; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+    if (lane == 0) {
+      s.rf[0][warp] = mf;
+      s.rf[1][warp] = mq;
+      s.rf[2][warp] = e;
+    }
+    __syncthreads();
+    cut_q = INFINITY;
+#pragma unroll
+    for (int w = 0; w < kSw; ++w) {
+      mf = fmaxf(mf, s.rf[0][w]);
+      mq = fmaxf(mq, s.rf[1][w]);
+      cut_q = fminf(cut_q, s.rf[1][w]);
+    }
+    float low = INFINITY;
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      float a = 0.0f;
+#pragma unroll
+      for (int w = g; w < kSw; w += 4)
+        a += s.rf[0][w] > -INFINITY ? s.rf[2][w] * exp2f((s.rf[0][w] - mf) * 1.44269504f) : 0.0f;
+      low = fminf(low, a);
+    }
+    cut_f = mf + logf(0.5f * (1.0f - p.alpha) * low * (4.0f / (kRuns * kS)));
+    if (n < kRuns * kS) cut_f = -INFINITY;
+    if (n < kRuns * kS || (long long)p.k_max * 400 > vocab) cut_q = -INFINITY;
+    __syncthreads();
+  }
+  const float af = (float)bin_origin(mf), aq = (float)bin_origin(mq);
+  const float m0 = mf > -INFINITY ? mf : 0.0f;  // reference of the guess
+
+  // ---- pass A (z_fp last: pass B reads it again) ----
+  int n_cand = 0;  // z_q candidates of this thread
+  if (cut_q > -INFINITY)
+    q.each([&](const float4& v, int u) {
+      const float m = max4(v);
+      mq = fmaxf(mq, m);
+      if (m >= cut_q) {
+        const float z[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (z[k] >= cut_q) {
+            if (n_cand < kTopCap) s.cand[n_cand][t] = (uint16_t)(4 * u + k);
+            ++n_cand;
+          }
+      }
+    });
+  // candidates that fit are counted from the lists, else in a pass of its own
+  const bool listed = __syncthreads_and(n_cand <= kTopCap) && cut_q > -INFINITY;
+  if (listed) {
+    float z[kTopCap];
+#pragma unroll
+    for (int c = 0; c < kTopCap; ++c) {
+      const int e = c < n_cand ? s.cand[c][t] : 0;
+      z[c] = c < n_cand ? __ldg(rq + q.index(t, e >> 2, e & 3)) : -INFINITY;
+    }
+#pragma unroll
+    for (int c = 0; c < kTopCap; ++c)
+      if (z[c] >= bin_floor(aq)) atomicAdd(&s.hq[bin_of(z[c], aq)], 1u);
+  } else {
+    const float low = bin_floor(aq);
+    q.each([&](const float4& v, int) {
+      mq = fmaxf(mq, max4(v));
+      const float z[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (z[k] >= low) atomicAdd(&s.hq[bin_of(z[k], aq)], 1u);
+    });
+  }
+  cut_f = fmaxf(cut_f, bin_floor(af));  // (NaN: the floor)
+  float guess = 0.0f;                   // S_fp times e^(m - m0), about
+  f.each([&](const float4& v, int) {
+    const float m = max4(v);
+    mf = fmaxf(mf, m);
+    const float z[4] = {v.x, v.y, v.z, v.w};
+    guess += (exp_guess(z[0], m0) + exp_guess(z[1], m0)) +
+             (exp_guess(z[2], m0) + exp_guess(z[3], m0));
+    if (m >= cut_f) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (z[k] >= cut_f) atomicAdd(&s.hf[bin_of(z[k], af)], 1u);
+    }
+  });
+  {
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+      mf = fmaxf(mf, __shfl_xor_sync(0xffffffffu, mf, o));
+      mq = fmaxf(mq, __shfl_xor_sync(0xffffffffu, mq, o));
+      guess += __shfl_xor_sync(0xffffffffu, guess, o);
+    }
+    if (lane == 0) {
+      s.rf[0][warp] = guess;
+      s.rf[1][warp] = mf;
+      s.rf[2][warp] = mq;
+    }
+    __syncthreads();
+    guess = 0.0f;
+#pragma unroll
+    for (int w = 0; w < kSw; ++w) {
+      guess += s.rf[0][w];
+      mf = fmaxf(mf, s.rf[1][w]);
+      mq = fmaxf(mq, s.rf[2][w]);
+    }
+    __syncthreads();
+  }
+
+  // ---- the plan ----
+  make_plan(s, m0, af, p.alpha * guess, (uint32_t)p.k_max);
+  const float y1 = kMagic + (float)s.pick[3], y2 = kMagic + (float)s.pick[4];
+  const float y3 = kMagic + (float)s.pick[8];
+  const bool planned = s.pick[7] != 0u && s.pick[9] != 0u;
+  __syncthreads();  // (the histograms and pick are free)
+  if (!planned) {
+    if (t == 0) m_t[row] = -1;
+    return;
+  }
+
+  // ---- pass B ----
+  Sums sums;
+  Fixed norm;
+  {
+    // z_q candidates down to its bin
+    auto list_q = [&](float z, int i) {
+      if (bin_place(z, aq) <= y3) {
+        const uint32_t pos = atomicAdd(&s.nq, 1u);
+        if (pos < (uint32_t)kL) s.lq[pos] = pack(fkey(z), (uint32_t)i);
+      }
+    };
+    // (the noted ones are all of them if even cut_q itself lies below the bin)
+    if (listed && bin_place(cut_q, aq) > y3) {
+      float z[kTopCap];
+#pragma unroll
+      for (int c = 0; c < kTopCap; ++c) {
+        const int e = c < n_cand ? s.cand[c][t] : 0;
+        z[c] = c < n_cand ? __ldg(rq + q.index(t, e >> 2, e & 3)) : -INFINITY;
+      }
+#pragma unroll
+      for (int c = 0; c < kTopCap; ++c)
+        if (c < n_cand) list_q(z[c], q.index(t, s.cand[c][t] >> 2, s.cand[c][t] & 3));
+    } else {
+      q.each([&](const float4& v, int u) {
+        if (bin_place(max4(v), aq) <= y3) {
+          list_q(v.x, q.index(t, u, 0));
+          list_q(v.y, q.index(t, u, 1));
+          list_q(v.z, q.index(t, u, 2));
+          list_q(v.w, q.index(t, u, 3));
+        }
+      });
+    }
+    int n_mem = 0;
+    // The noted members of the warp, laid side by side so that every lane has
+    // work: those above the bins into the sums, the others into the list.
+    auto flush = [&]() {
+      int at = n_mem;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, at, o);
+        if (lane >= o) at += x;
+      }
+      const int total = __shfl_sync(0xffffffffu, at, 31);
+      at -= n_mem;
+      for (int c = 0; c < n_mem; ++c)
+        s.flat[warp][at + c] = (uint16_t)((s.mem[c][t] << 5) | lane);  // (vector, element, lane)
+      __syncwarp();
+      for (int j0 = 0; j0 < total; j0 += 64) {
+        int i[2];
+        float z[2], w[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const int j = j0 + 32 * k + lane;
+          const int e = j < total ? s.flat[warp][j] : 0;
+          i[k] = j < total ? f.index((t & ~31) | (e & 31), e >> 7, (e >> 5) & 3) : -1;
+          z[k] = i[k] >= 0 ? __ldg(rf + i[k]) : -INFINITY;
+          w[k] = i[k] >= 0 ? __ldg(rq + i[k]) : -INFINITY;
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          if (i[k] < 0) continue;
+          if (bin_place(z[k], af) >= y1) {
+            const uint32_t pos = atomicAdd(&s.nf, 1u);
+            if (pos < (uint32_t)kL) s.lf[pos] = pack(fkey(z[k]), (uint32_t)i[k]);
+          } else {
+            ++sums.cnt;
+            sums.add(expf(z[k] - mf), expf(w[k] - mq));
+          }
+        }
+      }
+      __syncwarp();
+      n_mem = 0;
+    };
+    f.each([&](const float4& v, int u) {
+      const float z[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) norm.add(expf(z[k] - mf));
+      if (bin_place(max4(v), af) <= y2) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (bin_place(z[k], af) <= y2) s.mem[n_mem++][t] = (uint16_t)(4 * u + k);
+      }
+      if (__any_sync(0xffffffffu, n_mem > kMemCap - 4)) flush();
+    });
+    flush();
+  }
+  {  // the mass above the listed elements, and S_fp
+    u64 a = sums.A.value(), b = norm.value();
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+      a += __shfl_xor_sync(0xffffffffu, a, o);
+      b += __shfl_xor_sync(0xffffffffu, b, o);
+    }
+    if (lane == 0) {
+      s.su[warp] = a;
+      s.sv[warp] = b;
+    }
+  }
+  __syncthreads();
+
+  // ---- finish ----
+  u64 above = 0ull, sum_f = 0ull;
+#pragma unroll
+  for (int w = 0; w < kSw; ++w) {
+    above += s.su[w];
+    sum_f += s.sv[w];
+  }
+  const uint32_t nf = s.nf, nq = s.nq;
+  const double sf = (double)sum_f;
+  __syncthreads();
+  bool ok = nf <= (uint32_t)kL && nq <= (uint32_t)kL && nq >= (uint32_t)p.k_max;
+  if (ok) {
+    // prefix mass >= alpha S  <=>  prefix >= ceil(alpha S) in fixed point
+    find_boundary(s, (int)nf, above, (u64)ceil((double)p.alpha * sf), mf);
+    ok = s.pick[2] != 0u;
+  }
+  if (!ok) {
+    if (t == 0) m_t[row] = -1;
+    return;
+  }
+  Pick pf;
+  pf.all = false;
+  pf.key = s.pick[0];
+  pf.idx = s.pick[1];
+  const u64* top = s.top;  // TopK(z_q, k_max) first
+  if (nq <= (uint32_t)kS) {  // by rank
+    if ((t & ~31) < (int)nq) {
+      const u64 e = t < (int)nq ? s.lq[t] : 0ull;
+      int r = 0;
+#pragma unroll 8
+      for (uint32_t k = 0; k < nq; ++k) r += s.lq[k] > e;
+      if (t < (int)nq) s.top[r] = e;
+    }
+    __syncthreads();
+  } else {
+    sort_desc<kS>(s.lq, (int)nq);
+    top = s.lq;
+  }
+  // the listed members of C; the first `window` of TopK(z_q, k_max) are S
+  for (int j = t; j < (int)nf; j += kS) {
+    const u64 w = s.lf[j];
+    if (ranks_in(pk_key(w), pk_idx(w), pf)) {
+      ++sums.cnt;
+      sums.add(expf(fval(pk_key(w)) - mf), expf(__ldg(rq + pk_idx(w)) - mq));
+    }
+  }
+  if (t < p.k_max) {
+    const u64 w = top[t];
+    const uint32_t gi = pk_idx(w);
+    const float z = __ldg(rf + gi), a = expf(z - mf);
+    const bool in_c = ranks_in(fkey(z), gi, pf);
+    s.wsel[t] = in_c ? fix40(a) : 0ull;
+    if (t < p.window) {
+      if (in_c) sums.C = fix40(a);
+      else sums.add(a, expf(fval(pk_key(w)) - mq));
+    }
+  }
+  warp_sums(sums, s.part[warp]);
+  __syncthreads();
+  if (warp == 0) {
+    u64 cnt = 0ull, A = 0ull, B = 0ull, C = 0ull;
+    Df aa, ab, bb;
+    if (lane < kSw) {
+      const u64* w = s.part[lane];
+      cnt = w[0];
+      A = w[1];
+      B = w[2];
+      C = w[3];
+      aa = Df::unpack(w[4]);
+      ab = Df::unpack(w[5]);
+      bb = Df::unpack(w[6]);
+    }
+    __syncwarp();
+    warp_sums(cnt, A, B, C, aa, ab, bb, s.part[0]);
+    if (lane == 0) {
+      const u64* w = s.part[0];
+      write_row(row, (int32_t)w[0], w[1], w[2], w[3], sf, Df::unpack(w[4]), Df::unpack(w[5]),
+                Df::unpack(w[6]), p, m_t, c_t, d_loc, y_t);
+    }
+  } else if (warp == 1) {
+    write_curve(s.wsel, sf, row, p.k_max, cov);
+  }
+}
+
+// K_b: column means of cov over the rows and the smallest k whose mean reaches
+// rho_K (0 if none).  One CTA, or a cluster of 8 for more than 64
+// rows of every thread: a thread takes one column of every (CTAs kWinT /
+// k_max)-th row, sixteen loads in flight, and the partial sums are added in a
+// fixed order in fp64 (rows of a CTA, then CTAs).  A thread's own rows add up
+// in a compensated fp32 sum, good to 2^-46: fp64 additions and conversions run
+// at two a cycle and SM here (256 rows of 256: 43 us in one CTA with them, 11
+// in eight, and 41 when each thread walked all rows of a column).
+constexpr int kWinT = 1024;
+constexpr int kWinLoads = 16;
+__global__ void __launch_bounds__(kWinT)
+    drift_window_kernel(const float* __restrict__ cov, int rows, int k_max, float rho_k,
+                        float* __restrict__ mean_cov, int32_t* __restrict__ k_b) {
+  __shared__ double part[kWinT];
+  __shared__ double col[kMaxKcov];
+  __shared__ int best[kMaxKcov / 32];
+  const int t = threadIdx.x, rank = (int)blockIdx.x, ctas = (int)gridDim.x;  // one cluster
+  pdl_wait();
+  const int per = kWinT / k_max;  // rows per sweep of a CTA
+  const int step = per * ctas;
+  Cs sum;
+  if (t < per * k_max) {
+    const int k = t % k_max;
+    for (long long r = rank * per + t / k_max; r < rows; r += kWinLoads * step) {
+      float v[kWinLoads];
+#pragma unroll
+      for (int i = 0; i < kWinLoads; ++i)
+        v[i] = r + i * step < rows ? __ldg(cov + (r + i * step) * k_max + k) : 0.0f;
+#pragma unroll
+      for (int i = 0; i < kWinLoads; ++i) sum.add(v[i]);
+    }
+    part[t] = (double)sum.hi + (double)sum.lo;
+  }
+  __syncthreads();
+  if (t < k_max) {
+    double c = 0.0;
+    for (int i = 0; i < per; ++i) c += part[i * k_max + t];
+    col[t] = c;
+  }
+  cluster_sync();  // (one CTA: a block barrier)
+  int mine = 0x7fffffff;
+  if (rank == 0 && t < kMaxKcov) {
+    if (t < k_max) {
+      double total = 0.0;
+      for (int r = 0; r < ctas; ++r)
+        total += __longlong_as_double((long long)ld_peer_u64(peer_addr(&col[t], (uint32_t)r)));
+      const double mean = total / rows;
+      mean_cov[t] = (float)mean;
+      if (mean >= (double)rho_k) mine = t + 1;
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) mine = min(mine, __shfl_xor_sync(0xffffffffu, mine, o));
+    if ((t & 31) == 0) best[t >> 5] = mine;
+  }
+  cluster_sync();  // the columns are read
+  if (rank == 0 && t == 0) {
     int b = 0x7fffffff;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) b = min(b, best[w]);
+    for (int w = 0; w < kMaxKcov / 32; ++w) b = min(b, best[w]);
     *k_b = b == 0x7fffffff ? 0 : b;
   }
 }
@@ -1028,21 +1865,67 @@ int drift_max_vocab() { return kCl * kSlice; }
 int drift_max_kcov() { return kMaxKcov; }
 int drift_cap() { return kCap; }
 
+namespace {
+template <int kS>
+cudaError_t launch_stream(const float* z_fp, const float* z_q, int rows, int vocab,
+                          const kvq_drift_params& p, int32_t* m_t, float* c_t, float* d_loc,
+                          uint8_t* y_t, float* cov, cudaStream_t st) {
+  const cudaError_t e = cudaFuncSetAttribute(
+      drift_stream_kernel<kS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Ss<kS>));
+  if (e != cudaSuccess) return e;
+  drift_stream_kernel<kS><<<rows, kS, sizeof(Ss<kS>), st>>>(z_fp, z_q, vocab, p, m_t, c_t, d_loc,
+                                                           y_t, cov);
+  return cudaGetLastError();
+}
+}  // namespace
+
 cudaError_t launch_drift(const float* z_fp, const float* z_q, int rows, int vocab,
                          const kvq_drift_params& p, int32_t* m_t, float* c_t, float* d_loc,
                          uint8_t* y_t, float* cov, cudaStream_t st) {
-  const size_t smem = sizeof(Sm);
-  cudaError_t e = cudaFuncSetAttribute(drift_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(drift_general_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(Sm));
   if (e != cudaSuccess) return e;
-  drift_kernel<<<dim3(kCl, rows), kT, smem, st>>>(z_fp, z_q, vocab, p, m_t, c_t, d_loc, y_t, cov);
-  return cudaGetLastError();
+  // at most one row per SM: all of an SM's threads on it
+  e = rows <= sms ? launch_stream<1024>(z_fp, z_q, rows, vocab, p, m_t, c_t, d_loc, y_t, cov, st)
+                  : launch_stream<512>(z_fp, z_q, rows, vocab, p, m_t, c_t, d_loc, y_t, cov, st);
+  if (e != cudaSuccess) return e;
+  // the rows it leaves: usually none, so the launch overlaps its end
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const int clusters = sms / kCl > 0 ? sms / kCl : 1;
+  cfg.gridDim = dim3(kCl, rows < clusters ? rows : clusters);
+  cfg.blockDim = dim3(kT);
+  cfg.dynamicSmemBytes = sizeof(Sm);
+  cfg.stream = st;
+  return cudaLaunchKernelEx(&cfg, drift_general_kernel, z_fp, z_q, rows, vocab, p, m_t, c_t, d_loc,
+                            y_t, cov);
 }
 
 cudaError_t launch_drift_window(const float* cov, int rows, int k_max, float rho_k,
                                 float* mean_cov, int32_t* k_b, cudaStream_t st) {
-  drift_window_kernel<<<1, 256, 0, st>>>(cov, rows, k_max, rho_k, mean_cov, k_b);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  const int ctas = (long long)rows * k_max > 64 * kWinT ? kCl : 1;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = ctas;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = ctas > 1 ? 2 : 1;
+  cfg.gridDim = dim3(ctas);
+  cfg.blockDim = dim3(kWinT);
+  cfg.stream = st;
+  return cudaLaunchKernelEx(&cfg, drift_window_kernel, cov, rows, k_max, rho_k, mean_cov, k_b);
 }
 
 }  // namespace kvq
