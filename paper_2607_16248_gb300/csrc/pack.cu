@@ -173,11 +173,25 @@ __device__ __forceinline__ RowSrc make_src(const Dims& d, const kvq_cache& c, co
   return s;
 }
 
-// Blocks made only of new tokens (prefill): one warp per quarter of a block
-// (quantize_quarter: key channels 32 w .. 32 w + 31 and value group w),
-// reading the rows straight from the input, so no staging tile and no
-// shared-memory atomics; many small CTAs keep the loads of many blocks in
-// flight.  grid (blocks, hkv, batch_count) of 128 threads.
+// A block whose first tokens are in the ring (at most residual / 32 + 1 per
+// call and kv-head).  Out of line: the kernel's body stays the one of the
+// blocks made of new tokens only.
+template <int BK, int BV>
+__device__ __noinline__ void quantize_mixed_quarter(const RowSrc src, int j, int qi, char* page) {
+  quantize_quarter<BK, BV>(
+      [&](int t) { return reinterpret_cast<const __half*>(src.k(j * kGroup + t)); },
+      [&](int t) { return reinterpret_cast<const __half*>(src.v(j * kGroup + t)); }, qi, page);
+}
+
+// Every block that leaves the window in a call of more than 32 tokens: one
+// warp per quarter of a block (quantize_quarter: key channels 32 w .. 32 w +
+// 31 and value group w), reading the rows straight from the input (or the
+// ring), so no staging tile and no shared-memory atomics; many small CTAs
+// keep the loads of many blocks in flight.  The ring keeps its rows until the
+// append kernel behind this one.  grid (blocks, hkv, batch_count) of 128
+// threads.  (With the four or five blocks that begin in the ring left to the
+// append kernel, one after another in one CTA per kv-head, a 4099-token chunk
+// of 4 x 8 heads at 4 bits took 49 us; here they are CTAs like the others.)
 constexpr int kInputThreads = 4 * 32;
 
 template <int BK, int BV>
@@ -189,11 +203,15 @@ __global__ void __launch_bounds__(kInputThreads)
   const int L0 = c.seq_len[b];
   const int L1 = L0 + n_new;
   if (L1 > d.max_len) return;  // the append kernel reports the overflow
-  const int first = max(packed_len(L0, d.residual), ((L0 + kGroup - 1) / kGroup) * kGroup) / kGroup;
-  const int j = first + blockIdx.x;
+  const int j = packed_len(L0, d.residual) / kGroup + blockIdx.x;
   if (j >= packed_len(L1, d.residual) / kGroup) return;
   char* page = page_ptr(d, c, b, h, j);
   if (!page) return;
+  if (j * kGroup < L0) {
+    quantize_mixed_quarter<BK, BV>(make_src(d, c, k_new, v_new, n_new, b, bi, h, L0), j,
+                                   threadIdx.x >> 5, page);
+    return;
+  }
   const long long nh = ((long long)bi * d.hkv + h) * n_new;
   const __half* nk = k_new + (nh + (long long)j * kGroup - L0) * kHeadDim;
   const __half* nv = v_new + (nh + (long long)j * kGroup - L0) * kHeadDim;
@@ -225,8 +243,10 @@ cudaError_t launch_input_blocks(const Dims& d, cudaLaunchConfig_t& cfg, const kv
   }
 }
 
-// Blocks that touch the ring, the ring append, and the length update.
-// grid (hkv, batch_count); the last CTA of a sequence (ticket) publishes L1.
+// The ring append and the length update, and in calls of at most 32 tokens the
+// blocks that leave the window (all of them begin in the ring).  grid (hkv,
+// batch_count, parts), parts > 1 only in longer calls, whose ring rows they
+// share; the last CTA of a sequence (ticket) publishes L1.
 __global__ void __launch_bounds__(kPackThreads)
     pack_append_kernel(Dims d, kvq_cache c, const __half* __restrict__ k_new,
                        const __half* __restrict__ v_new, int n_new, int batch_begin) {
@@ -243,8 +263,9 @@ __global__ void __launch_bounds__(kPackThreads)
   const int Lq0 = packed_len(L0, d.residual), Lq1 = packed_len(L1, d.residual);
   const RowSrc src = make_src(d, c, k_new, v_new, n_new, b, bi, h, L0);
 
-  // 1. Groups leaving the window that start below L0 (they read the ring).
-  const int j_end = min(Lq1, ((L0 + kGroup - 1) / kGroup) * kGroup) / kGroup;
+  // 1. Groups leaving the window (they read the ring); longer calls have
+  // quantized them in pack_input_blocks_kernel.
+  const int j_end = n_new > kGroup ? 0 : Lq1 / kGroup;
   for (int j = Lq0 / kGroup; j < j_end; ++j) {
     char* page = page_ptr(d, c, b, h, j);
     if (!page) continue;
@@ -259,19 +280,20 @@ __global__ void __launch_bounds__(kPackThreads)
   __half* ring_k = reinterpret_cast<__half*>(c.k_resid) + bh * d.ring * kHeadDim;
   __half* ring_v = reinterpret_cast<__half*>(c.v_resid) + bh * d.ring * kHeadDim;
   const int p0 = max(Lq1, L0);
-  for (int e = threadIdx.x; e < (L1 - p0) * 16; e += kPackThreads) {
+  for (int e = blockIdx.z * kPackThreads + threadIdx.x; e < (L1 - p0) * 16;
+       e += gridDim.z * kPackThreads) {
     const int p = p0 + (e >> 4), piece = e & 15;
     reinterpret_cast<uint4*>(ring_k + (long long)(p % d.ring) * kHeadDim)[piece] = src.k(p)[piece];
     reinterpret_cast<uint4*>(ring_v + (long long)(p % d.ring) * kHeadDim)[piece] = src.v(p)[piece];
   }
 
-  // 3. Publish the new length once every kv-head of the sequence has read L0.
+  // 3. Publish the new length once every CTA of the sequence has read L0.
   __syncthreads();
   if (threadIdx.x == 0) {
     unsigned* tickets = reinterpret_cast<unsigned*>(c.seq_len) + d.batch + 2;
     __threadfence();
     const unsigned t = atomicAdd(&tickets[b], 1u);
-    if (t == (unsigned)d.hkv - 1) {
+    if (t == (unsigned)d.hkv * gridDim.z - 1u) {
       c.seq_len[b] = L1;
       tickets[b] = 0u;
       __threadfence();
@@ -300,7 +322,7 @@ cudaError_t launch_pack(const Dims& d, const kvq_cache& cache, const __half* k_n
     if (e != cudaSuccess) return e;
     cfg.blockDim = dim3(kPackThreads);
   }
-  cfg.gridDim = dim3(d.hkv, batch_count);
+  cfg.gridDim = dim3(d.hkv, batch_count, n_new > kGroup ? 4 : 1);
   e = cudaLaunchKernelEx(&cfg, pack_append_kernel, d, cache, k_new, v_new, n_new, batch_begin);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
