@@ -43,6 +43,8 @@
 
 #include <float.h>
 
+#include <atomic>
+
 #include "common.cuh"
 
 namespace kvq {
@@ -1095,7 +1097,7 @@ struct Ss {
   u64 wsel[kMaxKcov];             // coverage terms
   u64 part[kSw][8];               // warps' sums: count, A, B, C and S, saa, sab, sbb
   u64 su[kSw], sv[kSw];
-  float rf[3][kSw];
+  float rf[4][kSw];
   uint32_t sc[2][kSw];
   uint32_t pick[12];
   uint32_t nf, nq;                // list lengths
@@ -1273,23 +1275,31 @@ __device__ __forceinline__ T scan(T x, T* buf, T* total) {
   }
   if (l == 31) buf[w] = i;
   __syncthreads();
-  T before = 0, all = 0;
+  // (the warps' totals by shuffles: a loop over 32 of them in every thread is
+  // longer than the scan)
+  T y = l < kS / 32 ? buf[l] : (T)0;
 #pragma unroll
-  for (int v = 0; v < kS / 32; ++v) {
-    const T y = buf[v];
-    before += v < w ? y : (T)0;
-    all += y;
+  for (int o = 1; o < kS / 32; o <<= 1) {
+    const T z = __shfl_up_sync(0xffffffffu, y, o);
+    if (l >= o) y += z;
   }
-  *total = all;
-  return before + i - x;
+  *total = __shfl_sync(0xffffffffu, y, kS / 32 - 1);
+  const T before = __shfl_sync(0xffffffffu, y, w > 0 ? w - 1 : 0);
+  return (w > 0 ? before : (T)0) + i - x;
 }
 
 // The bins [b1, b2] of z_fp to list, around the place where the prefix mass
-// should reach `goal` (in units of e^top), into pick[3..4] (pick[7] = 1 if they hold at most kL
-// elements), and the bin of z_q where the count reaches k_max into pick[8]
-// (pick[9] = 1 if at most kL elements rank above or in it).
+// should reach `goal` (in units of e^top), into pick[3..4] (pick[7] = 1 if
+// they hold at most kL elements), and the bin of z_q where the count reaches
+// k_max into pick[8] (pick[9] = 1 if at most kL elements rank above or in it).
+// `counted` is the mass of the counted elements: the goal is met from the end
+// of the histogram, where many small terms per bin leave no error, and not
+// from its start, where one token can hold a third of the mass and its bin's
+// width is 0.8% of that (44 rows of 20772 tokens, alpha = 0.99: some rows went
+// to the general kernel).
 template <int kS>
-__device__ void make_plan(Ss<kS>& s, float top, float a_f, float goal, uint32_t k_max) {
+__device__ void make_plan(Ss<kS>& s, float top, float a_f, float goal, float counted,
+                          uint32_t k_max) {
   constexpr int kPer = kBins / kS;
   const int t = threadIdx.x;
   if (t < 12) s.pick[t] = t == 0 || t == 8 ? kBins : 0u;
@@ -1311,6 +1321,7 @@ __device__ void make_plan(Ss<kS>& s, float top, float a_f, float goal, uint32_t 
   uint32_t all_c, all_d;
   const float wb = scan<kS>(ws, s.rf[0], &all_w);
   uint32_t x = scan<kS>(cs, s.sc[0], &all_c), y = scan<kS>(ds, s.sc[1], &all_d);
+  goal += all_w - counted;
   {
     uint32_t b = kBins;  // the first bin whose prefix mass reaches the goal
     float q = wb;
@@ -1399,11 +1410,8 @@ __device__ void find_boundary(Ss<kS>& s, int n, u64 above, u64 target, float mf)
     s.sc[1][w] = hi;
   }
   __syncthreads();
-#pragma unroll
-  for (int v = 0; v < kS / 32; ++v) {
-    lo = min(lo, s.sc[0][v]);
-    hi = max(hi, s.sc[1][v]);
-  }
+  lo = __reduce_min_sync(0xffffffffu, l < kS / 32 ? s.sc[0][l] : 0xffffffffu);
+  hi = __reduce_max_sync(0xffffffffu, l < kS / 32 ? s.sc[1][l] : 0u);
   const int sh = n > 0 ? max(0, 22 - __clz(hi - lo)) : 0;  // (hi - lo) >> sh < 1024 = kL
   auto part_of = [&](u64 e) { return (hi - pk_key(e)) >> sh; };
   auto mass_of = [&](u64 e) { return fix40(expf(fval(pk_key(e)) - mf)); };
@@ -1503,22 +1511,24 @@ __global__ void __launch_bounds__(kS, 1024 / kS)
       s.rf[2][warp] = e;
     }
     __syncthreads();
-    cut_q = INFINITY;
+    // second level: lane = warp
+    const float mw = lane < kSw ? s.rf[0][lane] : -INFINITY;
+    const float qw = lane < kSw ? s.rf[1][lane] : -INFINITY;
+    cut_q = lane < kSw ? qw : INFINITY;
+    mf = mw;
+    mq = qw;
 #pragma unroll
-    for (int w = 0; w < kSw; ++w) {
-      mf = fmaxf(mf, s.rf[0][w]);
-      mq = fmaxf(mq, s.rf[1][w]);
-      cut_q = fminf(cut_q, s.rf[1][w]);
+    for (int o = 16; o; o >>= 1) {
+      mf = fmaxf(mf, __shfl_xor_sync(0xffffffffu, mf, o));
+      mq = fmaxf(mq, __shfl_xor_sync(0xffffffffu, mq, o));
+      cut_q = fminf(cut_q, __shfl_xor_sync(0xffffffffu, cut_q, o));
     }
-    float low = INFINITY;
+    // four sums over every fourth warp (xor 4, 8, 16), then their least
+    float low = mw > -INFINITY ? s.rf[2][lane] * exp2f((mw - mf) * 1.44269504f) : 0.0f;
 #pragma unroll
-    for (int g = 0; g < 4; ++g) {
-      float a = 0.0f;
-#pragma unroll
-      for (int w = g; w < kSw; w += 4)
-        a += s.rf[0][w] > -INFINITY ? s.rf[2][w] * exp2f((s.rf[0][w] - mf) * 1.44269504f) : 0.0f;
-      low = fminf(low, a);
-    }
+    for (int o = 16; o > 2; o >>= 1) low += __shfl_xor_sync(0xffffffffu, low, o);
+    low = fminf(low, __shfl_xor_sync(0xffffffffu, low, 1));
+    low = fminf(low, __shfl_xor_sync(0xffffffffu, low, 2));
     cut_f = mf + logf(0.5f * (1.0f - p.alpha) * low * (4.0f / (kRuns * kS)));
     if (n < kRuns * kS) cut_f = -INFINITY;
     if (n < kRuns * kS || (long long)p.k_max * 400 > vocab) cut_q = -INFINITY;
@@ -1566,17 +1576,22 @@ __global__ void __launch_bounds__(kS, 1024 / kS)
     });
   }
   cut_f = fmaxf(cut_f, bin_floor(af));  // (NaN: the floor)
-  float guess = 0.0f;                   // S_fp times e^(m - m0), about
+  float guess = 0.0f, counted = 0.0f;   // S_fp times e^(m - m0), about, and the counted part
   f.each([&](const float4& v, int) {
     const float m = max4(v);
     mf = fmaxf(mf, m);
     const float z[4] = {v.x, v.y, v.z, v.w};
-    guess += (exp_guess(z[0], m0) + exp_guess(z[1], m0)) +
-             (exp_guess(z[2], m0) + exp_guess(z[3], m0));
+    float e[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) e[k] = exp_guess(z[k], m0);
+    guess += (e[0] + e[1]) + (e[2] + e[3]);
     if (m >= cut_f) {
 #pragma unroll
       for (int k = 0; k < 4; ++k)
-        if (z[k] >= cut_f) atomicAdd(&s.hf[bin_of(z[k], af)], 1u);
+        if (z[k] >= cut_f) {
+          atomicAdd(&s.hf[bin_of(z[k], af)], 1u);
+          counted += e[k];
+        }
     }
   });
   {
@@ -1585,25 +1600,31 @@ __global__ void __launch_bounds__(kS, 1024 / kS)
       mf = fmaxf(mf, __shfl_xor_sync(0xffffffffu, mf, o));
       mq = fmaxf(mq, __shfl_xor_sync(0xffffffffu, mq, o));
       guess += __shfl_xor_sync(0xffffffffu, guess, o);
+      counted += __shfl_xor_sync(0xffffffffu, counted, o);
     }
     if (lane == 0) {
       s.rf[0][warp] = guess;
+      s.rf[3][warp] = counted;
       s.rf[1][warp] = mf;
       s.rf[2][warp] = mq;
     }
     __syncthreads();
-    guess = 0.0f;
+    guess = lane < kSw ? s.rf[0][lane] : 0.0f;
+    counted = lane < kSw ? s.rf[3][lane] : 0.0f;
+    mf = lane < kSw ? s.rf[1][lane] : -INFINITY;
+    mq = lane < kSw ? s.rf[2][lane] : -INFINITY;
 #pragma unroll
-    for (int w = 0; w < kSw; ++w) {
-      guess += s.rf[0][w];
-      mf = fmaxf(mf, s.rf[1][w]);
-      mq = fmaxf(mq, s.rf[2][w]);
+    for (int o = 16; o; o >>= 1) {
+      guess += __shfl_xor_sync(0xffffffffu, guess, o);
+      counted += __shfl_xor_sync(0xffffffffu, counted, o);
+      mf = fmaxf(mf, __shfl_xor_sync(0xffffffffu, mf, o));
+      mq = fmaxf(mq, __shfl_xor_sync(0xffffffffu, mq, o));
     }
     __syncthreads();
   }
 
   // ---- the plan ----
-  make_plan(s, m0, af, p.alpha * guess, (uint32_t)p.k_max);
+  make_plan(s, m0, af, p.alpha * guess, counted, (uint32_t)p.k_max);
   const float y1 = kMagic + (float)s.pick[3], y2 = kMagic + (float)s.pick[4];
   const float y3 = kMagic + (float)s.pick[8];
   const bool planned = s.pick[7] != 0u && s.pick[9] != 0u;
@@ -1714,11 +1735,11 @@ __global__ void __launch_bounds__(kS, 1024 / kS)
   __syncthreads();
 
   // ---- finish ----
-  u64 above = 0ull, sum_f = 0ull;
+  u64 above = lane < kSw ? s.su[lane] : 0ull, sum_f = lane < kSw ? s.sv[lane] : 0ull;
 #pragma unroll
-  for (int w = 0; w < kSw; ++w) {
-    above += s.su[w];
-    sum_f += s.sv[w];
+  for (int o = 16; o; o >>= 1) {
+    above += __shfl_xor_sync(0xffffffffu, above, o);
+    sum_f += __shfl_xor_sync(0xffffffffu, sum_f, o);
   }
   const uint32_t nf = s.nf, nq = s.nq;
   const double sf = (double)sum_f;
@@ -1866,6 +1887,19 @@ int drift_max_kcov() { return kMaxKcov; }
 int drift_cap() { return kCap; }
 
 namespace {
+// SMs of the current device (looked up once per device).
+cudaError_t sm_count(int* sms) {
+  static std::atomic<int> known[64];
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  *sms = dev < 64 ? known[dev].load(std::memory_order_relaxed) : 0;
+  if (*sms > 0) return cudaSuccess;
+  e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess && dev < 64) known[dev].store(*sms, std::memory_order_relaxed);
+  return e;
+}
+
 template <int kS>
 cudaError_t launch_stream(const float* z_fp, const float* z_q, int rows, int vocab,
                           const kvq_drift_params& p, int32_t* m_t, float* c_t, float* d_loc,
@@ -1882,9 +1916,8 @@ cudaError_t launch_stream(const float* z_fp, const float* z_q, int rows, int voc
 cudaError_t launch_drift(const float* z_fp, const float* z_q, int rows, int vocab,
                          const kvq_drift_params& p, int32_t* m_t, float* c_t, float* d_loc,
                          uint8_t* y_t, float* cov, cudaStream_t st) {
-  int dev = 0, sms = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  int sms = 0;
+  cudaError_t e = sm_count(&sms);
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(drift_general_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)sizeof(Sm));
