@@ -132,15 +132,32 @@ __device__ __forceinline__ uint32_t hsub1024(uint32_t x) {
 // 4*gid + j of a 32-channel group for values) from two packed words a, b (two
 // channels for keys, two tokens for values): v[j] = (f_j code_a, f_j code_b)
 // as fp16, exact.  inv(j) = 1 / f_j.
-template <int B>
+//
+// Codes of 2 bits (and 4 in the wide layout) are taken as they lie in the ten
+// mantissa bits of an fp16 number whose exponent field is zero: bit i of it is
+// 2^(i - 24), so a code at bit i is code 2^i 2^-24, exactly, and an operand
+// register is one AND, where OR-ing the code into the mantissa of 1024 and
+// subtracting 1024 (the other widths) takes one instruction more: 128 of about
+// 600 for a K2V2 block.  The MMA aligns a product by its operands' exponent
+// fields, so a code k bits below the top of the mantissa loses k bits of the
+// accumulator's alignment.  Left at the bottom of the mantissa that costs 100
+// times the error; so each code is moved to the top bits, or two bits below
+// them where that saves a shift.  Error of fp32 results against 64 bits,
+// relative, mean over query groups of 1, 2, 4 and 5 and four seeds at 6000
+// tokens: K2V2 2.61e-6 with the subtraction, 2.60e-6 without; K4V4 in groups
+// of 5: 3.42e-6 and 3.05e-6, but in groups of up to 4 heads 2.52e-6 and
+// 2.71e-6, so the narrow layout keeps the subtraction for 4 bits.  Ragged
+// batch of 16 (8k to 32k tokens, 8 heads, groups of 4), K2V2: 109 -> 89 us.
+constexpr float kSub = 16777216.0f;  // 2^24
+template <int B, bool kWide>
 struct Codes;
 
 // 1-bit codes are stored in fragment order (key1_bit / val1_bit): the word
 // w of a lane rotated left by 4 r holds, at bit 10 + 16 e + j, the code of
 // row j and half e of one fragment register, so each register is one AND
 // (an fp16 with a single exponent bit set: 2^-14, 2^-13, 2^-11, 2^-7).
-template <>
-struct Codes<1> {
+template <bool kWide>
+struct Codes<1, kWide> {
   __device__ static constexpr float inv(int j) {
     return j == 0 ? 16384.0f : j == 1 ? 8192.0f : j == 2 ? 2048.0f : 128.0f;
   }
@@ -158,20 +175,23 @@ struct Codes<1> {
 __device__ __forceinline__ uint32_t comp(const uint4& u, int i) {
   return i == 0 ? u.x : i == 1 ? u.y : i == 2 ? u.z : u.w;
 }
-template <>
-struct Codes<2> {
+template <bool kWide>
+struct Codes<2, kWide> {
   __device__ static constexpr float inv(int j) {
-    return j == 0 ? 1.0f : j == 1 ? 0.25f : j == 2 ? 0.0625f : 0.015625f;
+    return j == 0 || j == 2 ? kSub / 256.0f : kSub / 64.0f;
   }
   __device__ static int word(int gid) { return gid >> 2; }
   __device__ static void get(uint32_t a, uint32_t b, uint32_t sel, uint32_t (&v)[4]) {
-    const uint32_t x = __byte_perm(a, b, sel);  // the lane's byte -> bits 0..7 of each half
-#pragma unroll
-    for (int j = 0; j < 4; ++j) v[j] = hsub1024((x & (0x00030003u << (2 * j))) | 0x64006400u);
+    const uint32_t x = __byte_perm(a, b, sel);  // the lane's byte -> both bytes of each half
+    const uint32_t y = x * 16u;                 // (a multiplication: not on the AND's pipe)
+    v[0] = x & 0x03000300u;
+    v[1] = y & 0x00C000C0u;
+    v[2] = y & 0x03000300u;
+    v[3] = x & 0x00C000C0u;
   }
 };
 template <>
-struct Codes<4> {
+struct Codes<4, false> {
   __device__ static constexpr float inv(int j) { return (j & 1) ? 0.0625f : 1.0f; }
   __device__ static int word(int gid) { return gid >> 1; }
   __device__ static void get(uint32_t a, uint32_t b, uint32_t sel, uint32_t (&v)[4]) {
@@ -184,7 +204,20 @@ struct Codes<4> {
   }
 };
 template <>
-struct Codes<8> {
+struct Codes<4, true> {
+  __device__ static constexpr float inv(int j) { return (j & 1) ? kSub / 16.0f : kSub / 64.0f; }
+  __device__ static int word(int gid) { return gid >> 1; }
+  __device__ static void get(uint32_t a, uint32_t b, uint32_t sel, uint32_t (&v)[4]) {
+    const uint32_t x = __byte_perm(a, b, sel);            // the lane's 16 bits -> each half
+    const uint32_t y = __byte_perm(a, b, sel ^ 0x1111u);  // their bytes swapped
+    v[0] = (x * 64u) & 0x03C003C0u;
+    v[1] = x & 0x00F000F0u;
+    v[2] = (y * 64u) & 0x03C003C0u;
+    v[3] = y & 0x00F000F0u;
+  }
+};
+template <bool kWide>
+struct Codes<8, kWide> {
   __device__ static constexpr float inv(int) { return 1.0f; }
   __device__ static int word(int gid) { return gid; }
   __device__ static void get(uint32_t a, uint32_t b, uint32_t, uint32_t (&v)[4]) {
@@ -376,11 +409,11 @@ __device__ __forceinline__ void tc_unit(const char* const (&pg)[NB], const char*
       for (int half = 0; half < 2; ++half) {
         uint32_t v[4];
         if constexpr (BK == 1) {
-          Codes<1>::rot(comp(kw1[bi], ks >> 1), 2 * (ks & 1) + half, v);
+          Codes<1, kWide>::rot(comp(kw1[bi], ks >> 1), 2 * (ks & 1) + half, v);
         } else {
           const uint32_t wa = *reinterpret_cast<const uint32_t*>(kc + 4 * ((c + 2 * half) * BK + ln.wk));
           const uint32_t wb = *reinterpret_cast<const uint32_t*>(kc + 4 * ((c + 2 * half + 1) * BK + ln.wk));
-          Codes<BK>::get(wa, wb, ln.sel_k, v);
+          Codes<BK, kWide>::get(wa, wb, ln.sel_k, v);
         }
         a0[2 * half] = v[0];
         a0[2 * half + 1] = v[1];
@@ -438,7 +471,7 @@ __device__ __forceinline__ void tc_unit(const char* const (&pg)[NB], const char*
           const int j = 2 * mt + rh;
           const float d = dk[bi][mt][2 * rh + hh];
           const float full = kWide ? d : d + __shfl_xor_sync(0xffffffffu, d, 2);
-          sc[bi][j][hh] = fmaf(full, Codes<BK>::inv(j) * scale_log2, hh ? z1 : z0);
+          sc[bi][j][hh] = fmaf(full, Codes<BK, kWide>::inv(j) * scale_log2, hh ? z1 : z0);
         }
   }
 
@@ -475,7 +508,7 @@ __device__ __forceinline__ void tc_unit(const char* const (&pg)[NB], const char*
           for (int dl = 0; dl < 2; ++dl) {
             const int ia = 2 * ks + dl;
             uint32_t v[4];
-            Codes<1>::rot(comp(vw, g), ia, v);
+            Codes<1, kWide>::rot(comp(vw, g), ia, v);
             am0[2 * dl] = v[0];
             am0[2 * dl + 1] = v[1];
             am1[2 * dl] = v[2];
@@ -534,8 +567,8 @@ __device__ __forceinline__ void tc_unit(const char* const (&pg)[NB], const char*
         for (int dl = 0; dl < 2; ++dl) {
           const int ia = 2 * ks + dl, ib = ia + 4;  // tokens 8tig + ia, 8tig + ib
           uint32_t v[4];
-          if constexpr (BV == 1) Codes<1>::rot(comp(vw1, g), ia, v);
-          else Codes<BV>::get(cw[ia], cw[ib], ln.sel_v, v);
+          if constexpr (BV == 1) Codes<1, kWide>::rot(comp(vw1, g), ia, v);
+          else Codes<BV, kWide>::get(cw[ia], cw[ib], ln.sel_v, v);
           am0[2 * dl] = v[0];
           am0[2 * dl + 1] = v[1];
           am1[2 * dl] = v[2];
@@ -570,8 +603,8 @@ __device__ __forceinline__ Lane make_lane(int lane) {
   ln.tig = lane & 3;
   ln.sel_k = code_selector<BK>(ln.gid);
   ln.sel_v = code_selector<BV>(ln.gid);
-  ln.wk = Codes<BK>::word(ln.gid);
-  ln.wv = Codes<BV>::word(ln.gid);
+  ln.wk = Codes<BK, false>::word(ln.gid);
+  ln.wv = Codes<BV, false>::word(ln.gid);
   ln.neg_lo = ln.gid >= 4 ? 0xBC00BC00u : 0u;
   ln.p_lo = ln.tig >= 2 ? 1.0f : 0.0f;
   return ln;
@@ -645,7 +678,7 @@ __device__ __forceinline__ void tc_write_state(const TcState& st, WarpState& ws,
       for (int rh = 0; rh < 2; ++rh) {
         const int jp = 2 * half + rh;
         const int cch = kPacked ? 32 * g + 4 * gid + jp : 16 * mtp + gid + 8 * rh;
-        const float inv = kPacked ? Codes<BV>::inv(jp) : 1.0f;
+        const float inv = kPacked ? Codes<BV, kWide>::inv(jp) : 1.0f;
 #pragma unroll
         for (int hh = 0; hh < 2; ++hh) {
           const float a = st.acc[mtp][2 * rh + hh];
