@@ -727,25 +727,80 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
   }
   __syncwarp();
   // The plan reads the lengths many times: one coalesced read into shared
-  // memory after the dependency wait instead of global round trips.  (No
-  // copies are started before the wait: the next CTA of an SM starts only
-  // when the previous kernel's CTA there has left, so little would overlap,
-  // and the reads after the wait would queue behind them.)
-  const int* lens = d.batch <= kLenCap ? len_s : c.seq_len;
-  __syncthreads();  // zero rows written
-  pdl_wait();
-
-  // ---- the plan from the lengths after the wait ----
-  // (kept in shared memory: it is needed again only after the streaming)
-  if (d.batch <= kLenCap)
-    for (int b = threadIdx.x; b < d.batch; b += kThreads) len_s[b] = read_len(c.seq_len + b);
-  __syncthreads();
-  {
+  // memory instead of global round trips.
+  const bool short_batch = d.batch <= kLenCap;
+  const int* lens = short_batch ? len_s : c.seq_len;
+  const FlatGrid& g = grid_s;
+  int v = -1;  // this warp's virtual warp, -1 without work
+  // The plan from `lens`, and the walk of this warp (kept in shared memory:
+  // nothing of them holds registers across the streaming loop).
+  auto make_plan = [&]() {
     const FlatGrid g0 = flat_grid(plan_sums(lens, d, append), gridDim.x);
     if (threadIdx.x == 0) grid_s = g0;
+    __syncthreads();
+    v = (int)blockIdx.x < g.n_cta ? cta_first_v(blockIdx.x, g) + warp : -1;
+    if (v >= 0 && v >= cta_first_v(blockIdx.x + 1, g)) v = -1;
+    if (v >= 0) {
+      const long long a = v_first_unit(v, g);
+      const Walk w0 = walk_start(a, lens, d, append, g.k);
+      if (lane == 0) {
+        X.w = w0;
+        X.a = a;
+        X.e = v_first_unit(v + 1, g);
+        X.last_v = v == g.n_v - 1;
+      }
+      __syncwarp();
+    }
+  };
+  // Before the dependency wait: the plan for the lengths as they are now, and
+  // the warp's first slots of blocks that no kernel still writes (a page never
+  // changes once written; the newest block of each pair may be the one the
+  // previous kernel is writing).  The lengths are compared after the wait, and
+  // the plan is made again if one changed (early slots that its range does not
+  // begin with are consumed without use).  A CTA starts here when the previous
+  // kernel's CTA on its SM has left and then waits for the slowest of that
+  // kernel's (7 to 14 us in a chain of layers), so this hides the plan (2.3 to
+  // 3 us) and the first copies (about 1.5 us).
+  if (short_batch) {
+    for (int b = threadIdx.x; b < d.batch; b += kThreads) len_s[b] = read_len(c.seq_len + b);
+    __syncthreads();  // (and the zero rows are written)
+    make_plan();
+    if (v >= 0) {
+      const Walk w = X.w;
+      if (w.b < d.batch && w.pc > 0) {
+        const long long U = w.Ub + (long long)w.h * w.pc;
+        const PairShape s = pair_shape(w.L, d.residual);
+        const int j0 = min(items_below(X.a - U, s.nb, s.nr, g.k, w.f), s.nb);
+        const int j1 = min(items_below(X.e - U, s.nb, s.nr, g.k, w.f), s.nb);
+        TableWin tw;
+        table_win_init(tw);
+        int end = 0;
+        const int n = tc_pre_issue<BK, BV>(page_map(d, c, w.b, w.h), tw, j0, j1, s.nb - 1, ring,
+                                           full, R, end, flag);
+        if (lane == 0) {
+          X.pre = n;
+          X.pre_end = end;
+          X.lo_h = j0;
+          X.p_h = w.b * d.hkv + w.h;
+        }
+        __syncwarp();
+      }
+    }
   }
   __syncthreads();
-  const FlatGrid& g = grid_s;
+  pdl_wait();
+  bool stale = !short_batch;
+  if (short_batch) {
+    for (int b = threadIdx.x; b < d.batch; b += kThreads) stale |= read_len(c.seq_len + b) != len_s[b];
+    stale = __syncthreads_or(stale);
+  }
+  if (stale) {
+    if (short_batch) {
+      for (int b = threadIdx.x; b < d.batch; b += kThreads) len_s[b] = read_len(c.seq_len + b);
+      __syncthreads();
+    }
+    make_plan();
+  }
   if (g.N == 0 && blockIdx.x == 0 && warp == 0)
     for (int i = lane; i < P * gq * kHeadDim; i += 32) store_out(out, out_f16, i, 0.0f);
   // Early copies still in flight that no packed range consumed land before
@@ -794,19 +849,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 
   // The walk and the current segment live in shared memory (X): nothing of
   // them holds registers across the streaming loop, which gets them all.
-  const int v = (int)blockIdx.x < g.n_cta ? cta_first_v(blockIdx.x, g) + warp : -1;
-  if (v >= 0 && v < cta_first_v(blockIdx.x + 1, g)) {
-    {
-      const long long a = v_first_unit(v, g);
-      const Walk w0 = walk_start(a, lens, d, append, g.k);
-      if (lane == 0) {
-        X.w = w0;
-        X.a = a;
-        X.e = v_first_unit(v + 1, g);
-        X.last_v = v == g.n_v - 1;
-      }
-      __syncwarp();
-    }
+  if (v >= 0) {
     for (;;) {
       Walk w = X.w;
       if (w.b >= d.batch) break;
