@@ -89,6 +89,7 @@ __host__ __device__ inline Ws carve(void* base, int batch, int hq, int hkv, int 
 struct MergeSmall {
   float ww[kWarps][kHeads];             // warp merge weights 2^(m_w - M)
   float gm[kWarps][kHeads];             // a group's maximum M
+  float gl[kWarps][kHeads];             // a group's row sum
 };
 // The CTA's merge groups: warps [w0, w1) end in the same pair; cnt = the
 // pair's partials in all.
@@ -1011,38 +1012,44 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
   }
   __syncthreads();
   const int ng = mg.n;
-  if (threadIdx.x < ng) {  // a group's partial count, once (64-bit divisions)
-    const SegRec r = rec[mg.w0[threadIdx.x]];
+  // a group's partial count, once (64-bit divisions), in a warp that the
+  // weights below do not use (ng * gq <= 128 threads)
+  if (warp == kWarps - 1 && lane < ng) {
+    const SegRec r = rec[mg.w0[lane]];
     int c_a, n_cta;
     bool cont;
-    mg.cnt[threadIdx.x] = pair_partials(r.U, r.pc, r.nb, r.nr, r.f, g, c_a, n_cta, cont);
+    mg.cnt[lane] = pair_partials(r.U, r.pc, r.nb, r.nr, r.f, g, c_a, n_cta, cont);
   }
   if (threadIdx.x < ng * gq) {  // (group, head): maximum and warp weights
     const int k = threadIdx.x / gq, gg = threadIdx.x - k * gq;
     const int w0 = mg.w0[k], w1 = mg.w1[k];
-    float mw[kWarps];
-    float M = -INFINITY;
+    float mw[kWarps], lw[kWarps];
+    float M = -INFINITY, l = 0.0f;
 #pragma unroll
     for (int w = 0; w < kWarps; ++w) {  // independent loads, then the maximum
       mw[w] = w >= w0 && w < w1 ? wstate(w).m[gg] : -INFINITY;
+      lw[w] = w >= w0 && w < w1 ? wstate(w).l[gg] : 0.0f;
       M = fmaxf(M, mw[w]);
     }
 #pragma unroll
     for (int w = 0; w < kWarps; ++w)
-      if (w >= w0 && w < w1) ms.ww[w][gg] = mw[w] == -INFINITY ? 0.0f : fast_exp2(mw[w] - M);
+      if (w >= w0 && w < w1) {
+        const float wt = mw[w] == -INFINITY ? 0.0f : fast_exp2(mw[w] - M);
+        ms.ww[w][gg] = wt;
+        l = fmaf(wt, lw[w], l);
+      }
     ms.gm[k][gg] = M;
+    ms.gl[k][gg] = l;
   }
   __syncthreads();
   for (int it = threadIdx.x; it < ng * gq * kHeadDim; it += kThreads) {
     const int ch = it & (kHeadDim - 1), kg = it >> 7;  // kHeadDim == 128
     const int k = kg / gq, gg = kg - k * gq;
     const int w0 = mg.w0[k], w1 = mg.w1[k];
-    float o = 0.0f, l = 0.0f;
-    for (int w = w0; w < w1; ++w) {
-      const float wt = ms.ww[w][gg];
-      o = fmaf(wt, wstate(w).o[gg][ch], o);
-      l = fmaf(wt, wstate(w).l[gg], l);
-    }
+    float o = 0.0f;
+    const float l = ms.gl[k][gg];
+#pragma unroll 4
+    for (int w = w0; w < w1; ++w) o = fmaf(ms.ww[w][gg], wstate(w).o[gg][ch], o);
     const int pp = rec[w0].p;
     if (mg.cnt[k] == 1) {
       const long long head0 = (long long)(pp / d.hkv) * d.hq + (long long)(pp % d.hkv) * gq;
@@ -1056,10 +1063,14 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
       }
     }
   }
+  // The CTA's partial rows come before its tickets: the barrier, then the
+  // release of the atomic (cumulative).  The decode step's count of CTAs that
+  // are done with the lengths goes out in the same round.
   __syncthreads();
+  if (append && threadIdx.x == kThreads - 1)
+    pub_last = atom_add_acq_rel(&ws.tk[P], 1u) == gridDim.x - 1u;
   if (threadIdx.x < ng && mg.cnt[threadIdx.x] > 1) {
     const SegRec r = rec[mg.w0[threadIdx.x]];
-    __threadfence();  // cumulativity: the CTA's partial rows before the ticket
     if (atom_add_acq_rel(&ws.tk[r.p], 1u) == (unsigned)mg.cnt[threadIdx.x] - 1u) {
       const int i = atomicAdd(&fin_n, 1);
       if (i < kFinCap) fin[i] = r;
@@ -1067,29 +1078,22 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
   }
   __syncthreads();
 
+  // ---- the decode step publishes the new lengths once every CTA is here ----
+  // (none reads a length after its ticket)
+  if (append && pub_last) {
+    for (int b = threadIdx.x; b < d.batch; b += kThreads) {
+      const int L0 = read_len(c.seq_len + b);
+      if (L0 < d.max_len) c.seq_len[b] = L0 + 1;
+      else atomicOr(flag, (unsigned)KVQ_FLAG_OVERFLOW);
+    }
+    if (threadIdx.x == 0) ws.tk[P] = 0u;
+  }
+
   // ---- final merges of the pairs whose last partial came from this CTA ----
   const int nf = min(fin_n, kFinCap);
   for (int i = 0; i < nf; ++i)
     final_merge(fin[i], g, d, ws, out, out_f16, reinterpret_cast<float*>(smem),
                 (size_t)kWarps * wbytes);
-
-  // ---- the decode step publishes the new lengths once every CTA is done ----
-  if (append) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      __threadfence();
-      pub_last = atom_add_acq_rel(&ws.tk[P], 1u) == gridDim.x - 1u;
-    }
-    __syncthreads();
-    if (pub_last) {
-      for (int b = threadIdx.x; b < d.batch; b += kThreads) {
-        const int L0 = read_len(c.seq_len + b);
-        if (L0 < d.max_len) c.seq_len[b] = L0 + 1;
-        else atomicOr(flag, (unsigned)KVQ_FLAG_OVERFLOW);
-      }
-      if (threadIdx.x == 0) ws.tk[P] = 0u;
-    }
-  }
 }
 
 size_t smem_bytes(const Dims& d) {
