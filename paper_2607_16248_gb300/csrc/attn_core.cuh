@@ -692,8 +692,9 @@ __device__ __forceinline__ void tc_write_state(const TcState& st, WarpState& ws,
 
 
 // ---------------------------------------------------------------------------
-// Tensor-core path for the fp16 residual window: a warp stages the K rows of
-// a 32-token chunk in shared memory, scores them with ldmatrix-fed MMAs
+// Tensor-core path for the fp16 residual window (the flat plan, and the split
+// plan's short ranges, take 16-token units, further below): a warp stages the
+// K rows of a 32-token chunk in shared memory, scores them with ldmatrix-fed MMAs
 // (keys as A with tokens as rows), then stages the V rows in the same place
 // (values transposed, channels as rows).  Rows past the window are zero and
 // their scores -inf.
@@ -762,6 +763,52 @@ __device__ __forceinline__ void tc_resid_values(const __half* vs_s, const uint32
     }
 }
 
+
+// A 16-token unit of the window, K rows and V rows staged at once (kHalfRows
+// each, K first): one m-tile of scores, one k-step of values.
+constexpr int kHalfTok = kGroup / 2;
+
+template <bool kWide, bool kCompact>
+__device__ __forceinline__ void tc_resid_half(const __half* rows, int n_tok,
+                                              const uint32_t (&qb)[16], const Lane& ln,
+                                              float scale_log2, TcState& st) {
+  const int lane = threadIdx.x & 31;
+  const int mi = lane >> 3, r8 = lane & 7;
+  float dk[2][4] = {};
+#pragma unroll
+  for (int ks = 0; ks < 8; ++ks) {
+    uint32_t a[4];
+    ldsm_x4(a, rows + (8 * (mi & 1) + r8) * kResRow + 16 * ks + 8 * (mi >> 1));
+    mma16816(dk[ks & 1], a[0], a[1], a[2], a[3], qb[2 * ks], qb[2 * ks + 1]);
+  }
+  float sc[1][4][2];
+  const float me[2] = {m_offset(st.m[0]), m_offset(st.m[1])};
+#pragma unroll
+  for (int rh = 0; rh < 2; ++rh) {
+    const bool ok = ln.gid + 8 * rh < n_tok;
+#pragma unroll
+    for (int hh = 0; hh < 2; ++hh) {
+      const float d = dk[0][2 * rh + hh] + dk[1][2 * rh + hh];
+      sc[0][rh][hh] = ok ? fmaf(d, scale_log2, -me[hh]) : -INFINITY;
+      sc[0][2 + rh][hh] = -INFINITY;
+    }
+  }
+  uint32_t pt[1][2][2], pl[1][2][2];
+  tc_softmax<1, kWide, kCompact, true>(sc, st, ln, pt, pl);
+  const __half* vs = rows + kHalfTok * kResRow;
+#pragma unroll
+  for (int mtp = 0; mtp < 8; ++mtp) {
+    uint32_t a[4];
+    ldsm_x4_t(a, vs + (8 * (mi >> 1) + r8) * kResRow + 16 * mtp + 8 * (mi & 1));
+    mma16816(st.acc[mtp], a[0], a[1], a[2], a[3], pt[0][0][0], pt[0][0][1]);
+    if constexpr (kWide && !kCompact)
+      mma16816(st.acc[mtp], a[0], a[1], a[2], a[3], pl[0][0][0], pl[0][0][1]);
+  }
+}
+
+
+// Shared-memory page image of a block that leaves the window (decode step).
+__host__ __device__ constexpr int image_bytes(int page) { return (page + 127) / 128 * 128; }
 
 // Blocks per ring slot and slots per warp for a page size.
 __host__ __device__ constexpr int ring_blocks(int page) { return page <= 3072 ? 2 : 1; }
@@ -918,6 +965,38 @@ __device__ __forceinline__ bool stage_rows_bulk(__half* rows, const __half* ring
   __syncwarp();
   return ok;
 
+}
+
+// The same for a 16-token unit: K rows p0 .. p0 + 15 into `rows`, the V rows
+// behind them, one copy per lane.
+__device__ __forceinline__ bool stage_half_bulk(__half* rows, const __half* ring_k,
+                                                const __half* ring_v, int p0, int n_tok, int ring,
+                                                int p_new, const __half* k_row,
+                                                const __half* v_row, uint64_t* bar,
+                                                uint32_t parity) {
+  const int lane = threadIdx.x & 31, tok = lane & (kHalfTok - 1);
+  const bool is_v = lane >= kHalfTok;
+  __syncwarp();
+  if (tok >= n_tok) {
+    uint4* r = reinterpret_cast<uint4*>(rows + lane * kResRow);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) r[i] = make_uint4(0u, 0u, 0u, 0u);
+  }
+  if (lane == 0) {
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    mbar_expect_tx(bar, (uint32_t)(2 * n_tok * kHeadDim * 2));
+  }
+  __syncwarp();
+  if (tok < n_tok) {
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    const __half* src = p0 + tok == p_new
+                            ? (is_v ? v_row : k_row)
+                            : (is_v ? ring_v : ring_k) + (long long)((p0 + tok) % ring) * kHeadDim;
+    bulk_g2s(rows + lane * kResRow, src, kHeadDim * 2, bar);
+  }
+  const bool ok = __all_sync(0xffffffffu, mbar_wait(bar, parity));
+  __syncwarp();
+  return ok;
 }
 
 // One element of the attention output: the fp32 result, or its fp16

@@ -95,24 +95,31 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src, uint32_t 
                : "memory");
 }
 
-// Shared-memory page image of a block that leaves the window (decode step).
-__host__ __device__ constexpr int image_bytes(int page) { return (page + 127) / 128 * 128; }
 
 // ---------------------------------------------------------------------------
-// Work of one (sequence, kv-head): nb packed blocks and n_res window chunks
-// over NV warps.  The last n_resw warps take the window chunks (strided), the
-// other np warps contiguous block ranges whose sizes differ by at most one.
+// Work of one (sequence, kv-head): nb packed blocks and n_res units of the
+// window over NV warps.  The last n_resw warps take the window units (strided),
+// the other np warps contiguous block ranges whose sizes differ by at most one.
+// A unit is 32 tokens, staged in two round trips (K rows, then V rows in their
+// place), or 16 tokens whose K and V rows come together, on twice as many
+// warps.  The 16-token form is taken where the window warps end last: ranges
+// of at most two blocks (4k tokens, 8 heads, K2V2: 11.1 -> 10.2 us per layer),
+// and steps in which they also quantize a block that leaves the window (32k,
+// K1V1: 15.8 -> 14.2 us).  On longer ranges its extra window warps would be
+// missing from the blocks (1 to 4% slower at 3 to 14 blocks per warp).
 // ---------------------------------------------------------------------------
 
 struct Plan {
-  int Lq, nb, n_res, n_resw, np;
+  int Lq, nb, unit, n_res, n_resw, np;  // unit: tokens of a window unit
 };
 
-__host__ __device__ inline Plan make_plan(int L, int residual, int NV) {
+// `flush`: a block leaves the window in this kernel.
+__host__ __device__ inline Plan make_plan(int L, int residual, int NV, bool flush) {
   Plan p;
   p.Lq = packed_len(L, residual);
   p.nb = p.Lq / kGroup;
-  p.n_res = (L - p.Lq + kGroup - 1) / kGroup;
+  p.unit = flush || p.nb <= 2 * NV ? kHalfTok : kGroup;
+  p.n_res = (L - p.Lq + p.unit - 1) / p.unit;
   const int cap = p.nb == 0 ? NV : (NV / 4 > 1 ? NV / 4 : 1);
   p.n_resw = p.n_res < cap ? p.n_res : cap;
   p.np = NV - p.n_resw;
@@ -233,36 +240,49 @@ __device__ __forceinline__ void prefetch_rows_l2(const __half* ring_base, int p0
                  : "memory");
 }
 
-// Window warp: chunks c0, c0 + stride, ... of the fp16 window.
+// Window warp: units c0, c0 + stride, ... of the fp16 window; its state goes
+// to the start of its area.  Out of line, so that its registers do not count
+// against the block loop (inlined, 128k tokens at K4V4 took 1.7% longer).
 template <int BK, int BV, bool kWide>
-__device__ void tc_window_warp(const Dims& d, const __half* ring_k, const __half* ring_v,
-                               const Plan& p, int L, int c0, int stride, char* area,
-                               const __half* qh, int gq, float scale_log2, TcState& st,
-                               int p_new, const __half* k_row, const __half* v_row,
-                               uint64_t* bar, unsigned* flag) {
+__device__ __noinline__ void tc_window_warp(const Dims d, const __half* ring_k,
+                                            const __half* ring_v, const Plan p, int L, int c0,
+                                            int stride, char* area, const __half* qh, int gq,
+                                            float scale_log2, int p_new, const __half* k_row,
+                                            const __half* v_row, uint64_t* bar, unsigned* flag) {
+  TcState st;
+  init_state(st);
   const int lane = threadIdx.x & 31;
   const Lane ln = make_lane<BK, BV>(lane);
   uint32_t qb[16];
   load_qb<false, kWide>(qb, qh, gq, ln);
   __half* rows = reinterpret_cast<__half*>(area);
   uint32_t phase = 0u;
-  for (int u = c0; u < p.n_res; u += stride) {
-    const int p0 = p.Lq + u * kGroup;
-    const int n_tok = min(kGroup, L - p0);
-    uint32_t pt[1][2][2], pl[1][2][2];
-    if (!stage_rows_bulk(rows, ring_k, p0, n_tok, d.ring, p_new, k_row, bar, phase++ & 1u)) {
-      if ((threadIdx.x & 31) == 0) atomicOr(flag, KVQ_FLAG_WAIT_TIMEOUT);
-      return;
+  bool ok = true;
+  if (p.unit == kHalfTok) {
+    for (int u = c0; ok && u < p.n_res; u += stride) {
+      const int p0 = p.Lq + u * kHalfTok;
+      const int n_tok = min(kHalfTok, L - p0);
+      ok = stage_half_bulk(rows, ring_k, ring_v, p0, n_tok, d.ring, p_new, k_row, v_row, bar,
+                           phase++ & 1u);
+      if (ok) tc_resid_half<kWide, BV == 1>(rows, n_tok, qb, ln, scale_log2, st);
+      __syncwarp();
     }
-    tc_resid_scores<kWide, BV == 1>(rows, n_tok, qb, ln, scale_log2, st, pt, pl);
-    __syncwarp();
-    if (!stage_rows_bulk(rows, ring_v, p0, n_tok, d.ring, p_new, v_row, bar, phase++ & 1u)) {
-      if ((threadIdx.x & 31) == 0) atomicOr(flag, KVQ_FLAG_WAIT_TIMEOUT);
-      return;
+  } else {
+    for (int u = c0; ok && u < p.n_res; u += stride) {
+      const int p0 = p.Lq + u * kGroup;
+      const int n_tok = min(kGroup, L - p0);
+      uint32_t pt[1][2][2], pl[1][2][2];
+      ok = stage_rows_bulk(rows, ring_k, p0, n_tok, d.ring, p_new, k_row, bar, phase++ & 1u);
+      if (!ok) break;
+      tc_resid_scores<kWide, BV == 1>(rows, n_tok, qb, ln, scale_log2, st, pt, pl);
+      __syncwarp();
+      ok = stage_rows_bulk(rows, ring_v, p0, n_tok, d.ring, p_new, v_row, bar, phase++ & 1u);
+      if (ok) tc_resid_values<kWide, BV == 1>(rows, pt, pl, st);
+      __syncwarp();
     }
-    tc_resid_values<kWide, BV == 1>(rows, pt, pl, st);
-    __syncwarp();
   }
+  if (!ok && lane == 0) atomicOr(flag, KVQ_FLAG_WAIT_TIMEOUT);
+  tc_write_state<false, BV, kWide>(st, *reinterpret_cast<WarpState*>(area), lane);
 }
 
 
@@ -327,7 +347,9 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
     hint = __shfl_sync(0xffffffffu, hint, 0);
     if (append && hint < d.max_len) ++hint;  // the length this kernel will attend
     __syncwarp();
-    const Plan ph = make_plan(hint, d.residual, NV);
+    const bool hint_flush =
+        append && packed_len(hint, d.residual) > packed_len(hint - 1, d.residual);
+    const Plan ph = make_plan(hint, d.residual, NV, hint_flush);
     int lo_h = 0, hi_h = 0, pre = 0, pre_end = 0;
     if (v < ph.np) {
       block_range(ph, v, lo_h, hi_h);
@@ -345,15 +367,30 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
       // the newest token do not change; this is a hint, nothing waits on it)
       const int last = hint - (append ? 1 : 0) - 1;  // newest row not yet written
       for (int u = v - ph.np; u < ph.n_res; u += ph.n_resw) {
-        const int p0 = ph.Lq + u * kGroup;
-        const int n = min(kGroup, last - p0);
+        const int p0 = ph.Lq + u * ph.unit;
+        const int n = min(ph.unit, last - p0);
         if (n > 0) {
           prefetch_rows_l2(ring_k, p0, n, d.ring);
           prefetch_rows_l2(ring_v, p0, n, d.ring);
         }
       }
     }
-    __syncthreads();  // zero rows written
+    // A flush is folded in by the packed warp np - 1 (it owns the last block).
+    // The window warps of its CTA quantize the block's four quarters into the
+    // image while it streams (with no window warp in that CTA, its owner does
+    // them itself, before streaming).  (Before the dependency wait, as the flat
+    // plan does it, 32k at K1V1 took 7% longer.)
+    char* image = reinterpret_cast<char*>(smem + smem_size - 16 - kZeroBytes - image_bytes(page));
+    auto quantize_flush = [&](const Plan& pl, int blk) {
+      const int n_help = ((pl.np - 1) / kWarps + 1) * kWarps - pl.np;  // window warps in that CTA
+      if (n_help > 0 ? v < pl.np : v != pl.np - 1) return;
+      const int nw = n_help > 0 ? n_help : 1;
+      for (int qi = n_help > 0 ? v - pl.np : 0; qi < 4; qi += nw) {
+        flush_quarter<BK, BV>(ring_k, ring_v, blk * kGroup, d.ring, qi, image);
+        mbar_arrive(&fl_bar);
+      }
+    };
+    __syncthreads();  // zero rows written, barriers initialised
     pdl_wait();
     // q (written by the previous kernel) into shared memory while the length
     // is read: one round trip for both
@@ -385,24 +422,13 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
       if (lane < 16) reinterpret_cast<uint4*>(rk)[lane] = reinterpret_cast<const uint4*>(k_row)[lane];
       else reinterpret_cast<uint4*>(rv)[lane - 16] = reinterpret_cast<const uint4*>(v_row)[lane - 16];
     }
-    const bool same = L == hint;  // the plan made before the wait holds
-    const Plan p = same ? ph : make_plan(L, d.residual, NV);
-    const int flush_blk = grew && p.Lq > packed_len(L0, d.residual) ? p.nb - 1 : -1;
+    const bool flush = grew && packed_len(L, d.residual) > packed_len(L0, d.residual);
+    // the plan made before the wait holds (it took a step that grows if append)
+    const bool same = L == hint && grew == append;
+    const Plan p = same ? ph : make_plan(L, d.residual, NV, flush);
+    const int flush_blk = flush ? p.nb - 1 : -1;
     const bool packed = v < p.np;
-    // A flush is folded in by the packed warp np - 1 (it owns the last
-    // block).  The window warps of its CTA quantize the block's four quarters
-    // into the image while it streams; with no window warp in that CTA it
-    // does them itself, before streaming.
-    char* image = reinterpret_cast<char*>(smem + smem_size - 16 - kZeroBytes - image_bytes(page));
-    const int cta_f = (p.np - 1) / kWarps;
-    const int n_help = (cta_f + 1) * kWarps - p.np;  // window warps in CTA cta_f
-    if (flush_blk >= 0 && (int)blockIdx.x == cta_f && (n_help > 0 ? !packed : v == p.np - 1)) {
-      const int nw = n_help > 0 ? n_help : 1;
-      for (int qi = n_help > 0 ? v - p.np : 0; qi < 4; qi += nw) {
-        flush_quarter<BK, BV>(ring_k, ring_v, flush_blk * kGroup, d.ring, qi, image);
-        mbar_arrive(&fl_bar);
-      }
-    }
+    if (flush_blk >= 0 && (int)blockIdx.x == (p.np - 1) / kWarps) quantize_flush(p, flush_blk);
     TcState st;
     init_state(st);
     if (packed || pre > 0) {
@@ -416,13 +442,12 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
                              reinterpret_cast<const char*>(zero), q_s, gq, scale_log2, flag, st,
                              flush_blk, &fl_bar, image);
     }
-    if (!packed)
-      tc_window_warp<BK, BV, kWide>(d, ring_k, ring_v, p, L, v - p.np, p.n_resw, ring, q_s, gq,
-                             scale_log2, st, grew ? L0 : -1, k_row, v_row, &wbar[warp], flag);
     // the warp's ring is idle now: its state goes to the start of it
-    WarpState& mine = *reinterpret_cast<WarpState*>(ring);
-    if (packed) tc_write_state<true, BV, kWide>(st, mine, lane);
-    else tc_write_state<false, BV, kWide>(st, mine, lane);
+    if (packed)
+      tc_write_state<true, BV, kWide>(st, *reinterpret_cast<WarpState*>(ring), lane);
+    else
+      tc_window_warp<BK, BV, kWide>(d, ring_k, ring_v, p, L, v - p.np, p.n_resw, ring, q_s, gq,
+                                    scale_log2, grew ? L0 : -1, k_row, v_row, &wbar[warp], flag);
   }
   __syncthreads();
 
