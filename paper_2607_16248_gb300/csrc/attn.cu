@@ -100,8 +100,8 @@ struct MergeGroups {
 
 // ---------------------------------------------------------------------------
 // The flat work plan.  Pair p = b * Hkv + h (sequence b, kv-head h) is a list
-// of items: its packed 32-token blocks (cost 1 each), then the 32-token
-// chunks of its fp16 window (cost cw each); the first item costs sc more (a
+// of items: its packed 32-token blocks (cost 1 each), then the 16-token
+// units of its fp16 window (cost cw each); the first item costs sc more (a
 // warp that starts a pair waits once for its first pages).  All pairs' items
 // lie end to end in cost units, cut into n_v equal contiguous unit ranges,
 // one per virtual warp; an item belongs to the virtual warp whose range holds
@@ -123,8 +123,10 @@ struct MergeGroups {
 // written out directly.
 // ---------------------------------------------------------------------------
 
-// Cost weights: a window chunk costs cw units, the first item of a pair sc
-// more (measured: a chunk takes ~4 blocks' time, a pair start ~1), and the
+// Cost weights: a window unit costs cw units, the first item of a pair sc
+// more (measured: about 2 to 4 blocks' time, a pair start ~1; with 1, 2 and
+// 4 units the ragged batch below took 372, 337 and 330 us for four layers, and
+// 8 x 64k K1V1 414, 386 and 385), and the
 // block that leaves the window in a decode step fu more (its warp quantizes
 // the block alone; Mistral-7B shape, K2V2, ragged batch of 16 where some
 // sequence flushes on most steps: 0, 4, 8 and 12 units gave 4.30, 4.24,
@@ -137,13 +139,13 @@ struct Costs {
 };
 
 struct PairShape {
-  int Lq, nb, nr;  // packed tokens, packed blocks, window chunks
+  int Lq, nb, nr;  // packed tokens, packed blocks, window units
 };
 __host__ __device__ inline PairShape pair_shape(int L, int residual) {
   PairShape s;
   s.Lq = packed_len(L, residual);
   s.nb = s.Lq / kGroup;
-  s.nr = (L - s.Lq + kGroup - 1) / kGroup;
+  s.nr = (L - s.Lq + kGroup / 2 - 1) / (kGroup / 2);
   return s;
 }
 // Extra units f of a pair whose last packed block leaves the window in this
@@ -179,7 +181,7 @@ __host__ __device__ inline int items_below(long long x, int nb, int nr, Costs k,
   return c;
 }
 
-// Work totals of a launch: packed blocks, window chunks, non-empty pairs,
+// Work totals of a launch: packed blocks, window units, non-empty pairs,
 // pairs with a block leaving the window.
 struct WorkSums {
   long long nb, nr, np, nf;
@@ -216,7 +218,7 @@ __host__ __device__ inline FlatGrid flat_grid(const WorkSums& w, int ctas) {
   const long long cap = (long long)kWarps * ctas;
   // the heaviest weights under which every one of the cap warps can still
   // hold an item start (each range >= the largest item cost)
-  const Costs pick[3] = {{4, 1, 12}, {2, 1, 6}, {1, 0, 0}};
+  const Costs pick[3] = {{4, 1, 12}, {1, 1, 6}, {1, 0, 0}};
   int i = 0;
   for (; i < 2; ++i) {
     const long long N = w.nb + pick[i].cw * w.nr + pick[i].sc * w.np + pick[i].fu * w.nf;
@@ -496,13 +498,15 @@ __device__ __forceinline__ void prefetch_rows_l2(const __half* ring_base, int p0
                  : "memory");
 }
 
-// Window chunks [i0, i1) of one pair (chunk u = tokens Lq + 32 u ...), staged
-// in the warp's (idle) ring; *phase_io is the parity count of the warp's
-// staging barrier, kept across calls.  A bounded wait that gives up sets
-// KVQ_FLAG_WAIT_TIMEOUT and ends the chunks.
+// Window units [i0, i1) of one pair (unit u = tokens Lq + 16 u ...), K and V
+// rows staged together in the warp's (idle) ring; *phase_io is the parity
+// count of the warp's staging barrier, kept across calls.  A bounded wait that
+// gives up sets KVQ_FLAG_WAIT_TIMEOUT and ends them.  (32-token chunks, whose
+// V rows waited for the K rows' place, made one item of two round trips: in a
+// launch with little work the warps that held one ended last.)
 // Out of line, like tc_packed_warp.
 template <int BK, int BV, bool kWide>
-__device__ __noinline__ TcState tc_window_chunks(TcState st, const Dims d, const __half* ring_k,
+__device__ __noinline__ TcState tc_window_units(TcState st, const Dims d, const __half* ring_k,
                                                  const __half* ring_v, int Lq, int L, int i0,
                                                  int i1, char* area, const __half* qh, int gq,
                                                  float scale_log2, int p_new,
@@ -516,20 +520,14 @@ __device__ __noinline__ TcState tc_window_chunks(TcState st, const Dims d, const
   load_qb<false, kWide>(qb, qh, gq, ln);
   __half* rows = reinterpret_cast<__half*>(area);
   for (int u = i0; u < i1; ++u) {
-    const int p0 = Lq + u * kGroup;
-    const int n_tok = min(kGroup, L - p0);
-    uint32_t pt[1][2][2], pl[1][2][2];
-    if (!stage_rows_bulk(rows, ring_k, p0, n_tok, d.ring, p_new, k_row, bar, phase++ & 1u)) {
+    const int p0 = Lq + u * kHalfTok;
+    const int n_tok = min(kHalfTok, L - p0);
+    if (!stage_half_bulk(rows, ring_k, ring_v, p0, n_tok, d.ring, p_new, k_row, v_row, bar,
+                         phase++ & 1u)) {
       if (lane == 0) atomicOr(flag, KVQ_FLAG_WAIT_TIMEOUT);
       break;
     }
-    tc_resid_scores<kWide, BV == 1>(rows, n_tok, qb, ln, scale_log2, st, pt, pl);
-    __syncwarp();
-    if (!stage_rows_bulk(rows, ring_v, p0, n_tok, d.ring, p_new, v_row, bar, phase++ & 1u)) {
-      if (lane == 0) atomicOr(flag, KVQ_FLAG_WAIT_TIMEOUT);
-      break;
-    }
-    tc_resid_values<kWide, BV == 1>(rows, pt, pl, st);
+    tc_resid_half<kWide, BV == 1>(rows, n_tok, qb, ln, scale_log2, st);
     __syncwarp();
   }
   *phase_io = phase;
@@ -607,6 +605,35 @@ __device__ void final_merge(const SegRec& r, const FlatGrid& g, const Dims& d, c
   const long long s0 = (long long)c_a + r.p;       // first CTA slot
   const long long sw = warp_slot(gridDim.x, P, r.p);
   auto slot = [&](int k) -> long long { return k < n_cta ? s0 + k : sw; };
+  const long long head0 = (long long)(r.p / d.hkv) * d.hq + (long long)(r.p % d.hkv) * gq;
+  // Few partials (the usual case: a pair spans a few CTAs): each thread loads
+  // its column and the maxima and sums of its head in one round and needs no
+  // barrier (2 us less at the end of a launch than the staged form below).
+  constexpr int kFew = 8;
+  if (cnt <= kFew) {
+    for (int it = threadIdx.x; it < rows; it += kThreads) {
+      const int gg = it / kHeadDim;
+      float m[kFew], l[kFew], v[kFew];
+#pragma unroll
+      for (int k = 0; k < kFew; ++k) {
+        m[k] = k < cnt ? __ldcg(ws.m + slot(k) * gq + gg) : -INFINITY;
+        l[k] = k < cnt ? __ldcg(ws.l + slot(k) * gq + gg) : 0.0f;
+        v[k] = k < cnt ? __ldcg(ws.o + slot(k) * rows + it) : 0.0f;
+      }
+      float M = -INFINITY, Ls = 0.0f, o = 0.0f;
+#pragma unroll
+      for (int k = 0; k < kFew; ++k) M = fmaxf(M, m[k]);
+#pragma unroll
+      for (int k = 0; k < kFew; ++k) {
+        const float w = m[k] == -INFINITY ? 0.0f : exp2f(m[k] - M);
+        Ls = fmaf(w, l[k], Ls);
+        o = fmaf(w, v[k], o);
+      }
+      store_out(out, out_f16, head0 * kHeadDim + it, Ls > 0.0f ? o / Ls : 0.0f);
+    }
+    if (threadIdx.x == 0) ws.tk[r.p] = 0u;
+    return;
+  }
   for (int i = threadIdx.x; i < gq * cnt; i += kThreads) {
     const int gg = i / cnt, k = i % cnt;
     wv[i] = __ldcg(ws.m + slot(k) * gq + gg);
@@ -638,7 +665,6 @@ __device__ void final_merge(const SegRec& r, const FlatGrid& g, const Dims& d, c
     if (lane == 0) lsum[gg] = Ls;
   }
   __syncthreads();
-  const long long head0 = (long long)(r.p / d.hkv) * d.hq + (long long)(r.p % d.hkv) * gq;
   for (int it = threadIdx.x; it < rows; it += kThreads) {
     const int gg = it / kHeadDim;
     float o = 0.0f;
@@ -661,7 +687,7 @@ struct WarpCtx {
   Walk w;                        // the pair the walk is at
   SegRec seg;                    // the segment being folded
   long long a, e;                // the warp's unit range
-  int i0, i1;                    // the segment's window chunks
+  int i0, i1;                    // the segment's window units
   int last, last_v;              // the segment ends the range; last virtual warp
   int pre, pre_end, lo_h, p_h;   // early copies: count, end block, first block, pair
   int pos;                       // ring slots used
@@ -778,6 +804,14 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
         int end = 0;
         const int n = tc_pre_issue<BK, BV>(page_map(d, c, w.b, w.h), tw, j0, j1, s.nb - 1, ring,
                                            full, R, end, flag);
+        // rows of a block that leaves the window here (old, unchanging) into
+        // L2: this warp quantizes them
+        if (lane == 0 && w.L > w.L0 && s.Lq > packed_len(w.L0, d.residual) && j1 == s.nb &&
+            j1 > j0) {
+          const long long ro = ((long long)w.b * d.hkv + w.h) * d.ring * kHeadDim;
+          prefetch_rows_l2(reinterpret_cast<const __half*>(c.k_resid) + ro, s.Lq - kGroup, kGroup, d.ring);
+          prefetch_rows_l2(reinterpret_cast<const __half*>(c.v_resid) + ro, s.Lq - kGroup, kGroup, d.ring);
+        }
         if (lane == 0) {
           X.pre = n;
           X.pre_end = end;
@@ -893,8 +927,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
         if (i1 > i0 && lane == 0) {
           // window rows into L2 while the packed blocks stream (a hint; the
           // newest row is not written yet)
-          const int p0 = s.Lq + i0 * kGroup;
-          const int n = min(w.L, s.Lq + i1 * kGroup) - (grew ? 1 : 0) - p0;
+          const int p0 = s.Lq + i0 * kHalfTok;
+          const int n = min(w.L, s.Lq + i1 * kHalfTok) - (grew ? 1 : 0) - p0;
           if (n > 0) {
             prefetch_rows_l2(ring_k, p0, n, d.ring);
             prefetch_rows_l2(ring_v, p0, n, d.ring);
@@ -943,7 +977,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
             }
           }
           if (X.i1 > X.i0) {
-            // the window chunks continue this state in their own layout
+            // the window units continue this state in their own layout
             WarpState& t = *reinterpret_cast<WarpState*>(ring);
             tc_write_state<true, BV, kWide>(st, t, lane);
             __syncwarp();
@@ -960,7 +994,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
           const long long bh2 = (long long)wr.b * d.hkv + wr.h;
           const PairShape s2 = pair_shape(wr.L, d.residual);
           const bool grew2 = wr.L > wr.L0;
-          st = tc_window_chunks<BK, BV, kWide>(
+          st = tc_window_units<BK, BV, kWide>(
               st, d, reinterpret_cast<const __half*>(c.k_resid) + bh2 * d.ring * kHeadDim,
               reinterpret_cast<const __half*>(c.v_resid) + bh2 * d.ring * kHeadDim, s2.Lq, wr.L,
               X.i0, X.i1, ring, q + ((long long)wr.b * d.hq + (long long)wr.h * gq) * kHeadDim, gq,
