@@ -448,20 +448,27 @@ __device__ __forceinline__ TcState tc_packed_warp(TcState st, const PageMap pm, 
 // The block `blk` of a pair leaves the window in this kernel (decode step)
 // and has no page yet: the warp quantizes it from the fp16 ring rows exactly
 // as kvq_pack does (quantize_quarter, common.cuh) into its idle ring (or the
-// second page of the held tail unit), writes the page and folds it, with the
+// second page of the held tail unit), unless that was done before the
+// dependency wait (`ready`: the image), writes the page and folds it, with the
 // tail unit if there is one.  Rare (one block in 32 steps), so out of line.
 template <int BK, int BV, bool kWide>
 __device__ __noinline__ TcState tc_fold_flush(TcState st, const PageMap pm, int blk,
                                               const char* tail, char* ring, const char* zero,
                                               const __half* qh, int gq, float scale_log2,
                                               unsigned* flag, const __half* ring_k,
-                                              const __half* ring_v, int ring_len) {
+                                              const __half* ring_v, int ring_len,
+                                              char* ready) {
   constexpr int page = page_bytes_c(BK, BV);
   const int lane = threadIdx.x & 31;
   TableWin tw;
   table_win_init(tw);
-  char* img = tail ? const_cast<char*>(tail) + page : ring;
-  for (int qi = 0; qi < 4; ++qi) flush_quarter<BK, BV>(ring_k, ring_v, blk * kGroup, ring_len, qi, img);
+  char* img = tail ? const_cast<char*>(tail) + page : ready ? ready : ring;
+  if (!ready) {
+    for (int qi = 0; qi < 4; ++qi) flush_quarter<BK, BV>(ring_k, ring_v, blk * kGroup, ring_len, qi, img);
+  } else if (img != ready) {  // beside the tail page
+    for (int i = lane; i < page / 16; i += 32)
+      reinterpret_cast<uint4*>(img)[i] = reinterpret_cast<const uint4*>(ready)[i];
+  }
   __syncwarp();
   char* dst = const_cast<char*>(block_addr(pm, tw, blk));
   if (dst) {
@@ -691,6 +698,7 @@ struct WarpCtx {
   int last, last_v;              // the segment ends the range; last virtual warp
   int pre, pre_end, lo_h, p_h;   // early copies: count, end block, first block, pair
   int pos;                       // ring slots used
+  int img_p;                     // pair whose flushed block this warp holds as an image, or -1
   uint32_t wphase;               // window staging barrier parity count
   int j1;                        // the segment's end block
 };
@@ -710,6 +718,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
   __shared__ SegRec rec[kWarps];                  // each warp's final state (p < 0: none)
   __shared__ SegRec fin[kFinCap];                 // pairs whose partials this CTA completed
   __shared__ int fin_n;
+  __shared__ int image_taken;                     // the CTA's image of a flushed block is in use
   __shared__ int pub_last;
   __shared__ WarpCtx wctx[kWarps];                // each warp's walk and segment
   __shared__ FlatGrid grid_s;                     // the plan's grid
@@ -733,7 +742,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
   for (int i = threadIdx.x; i < kZeroBytes / 4; i += kThreads)
     zero[i] = i >= kOnesWord0 && i < kOnesWord0 + 16 ? 0x3C003C00u : 0u;
   unsigned* flag = reinterpret_cast<unsigned*>(c.seq_len) + d.batch;
-  if (threadIdx.x == 0) fin_n = 0;
+  if (threadIdx.x == 0) fin_n = image_taken = 0;
+  char* image = reinterpret_cast<char*>(smem + smem_size - 16 - kZeroBytes - image_bytes(page));
   if (lane == 0) {
     for (int i = 0; i < R; ++i) mbar_init(full + i, 1);
     mbar_init(&wbar[warp], 1);
@@ -749,6 +759,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
     X.lo_h = -1;
     X.p_h = -1;
     X.pos = 0;
+    X.img_p = -1;
     X.wphase = 0u;
     X.last = 0;
   }
@@ -804,13 +815,20 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
         int end = 0;
         const int n = tc_pre_issue<BK, BV>(page_map(d, c, w.b, w.h), tw, j0, j1, s.nb - 1, ring,
                                            full, R, end, flag);
-        // rows of a block that leaves the window here (old, unchanging) into
-        // L2: this warp quantizes them
-        if (lane == 0 && w.L > w.L0 && s.Lq > packed_len(w.L0, d.residual) && j1 == s.nb &&
-            j1 > j0) {
-          const long long ro = ((long long)w.b * d.hkv + w.h) * d.ring * kHeadDim;
-          prefetch_rows_l2(reinterpret_cast<const __half*>(c.k_resid) + ro, s.Lq - kGroup, kGroup, d.ring);
-          prefetch_rows_l2(reinterpret_cast<const __half*>(c.v_resid) + ro, s.Lq - kGroup, kGroup, d.ring);
+        // A block that leaves the window here: its rows are at least
+        // `residual` tokens old, so the first warp of the CTA that owns one
+        // quantizes it now into the CTA's image (used if the lengths hold).
+        if (w.L > w.L0 && s.Lq > packed_len(w.L0, d.residual) && j1 == s.nb && j1 > j0) {
+          int taken = 1;
+          if (lane == 0) taken = atomicExch(&image_taken, 1);
+          if (__shfl_sync(0xffffffffu, taken, 0) == 0) {
+            const long long ro = ((long long)w.b * d.hkv + w.h) * d.ring * kHeadDim;
+            for (int qi = 0; qi < 4; ++qi)
+              flush_quarter<BK, BV>(reinterpret_cast<const __half*>(c.k_resid) + ro,
+                                    reinterpret_cast<const __half*>(c.v_resid) + ro,
+                                    s.Lq - kGroup, d.ring, qi, image);
+            if (lane == 0) X.img_p = w.b * d.hkv + w.h;
+          }
         }
         if (lane == 0) {
           X.pre = n;
@@ -830,6 +848,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
     stale = __syncthreads_or(stale);
   }
   if (stale) {
+    if (lane == 0) X.img_p = -1;
     if (short_batch) {
       for (int b = threadIdx.x; b < d.batch; b += kThreads) len_s[b] = read_len(c.seq_len + b);
       __syncthreads();
@@ -973,7 +992,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
                   reinterpret_cast<const char*>(zero),
                   q + ((long long)wf.b * d.hq + (long long)wf.h * gq) * kHeadDim, gq, scale_log2,
                   flag, reinterpret_cast<const __half*>(c.k_resid) + bhf * d.ring * kHeadDim,
-                  reinterpret_cast<const __half*>(c.v_resid) + bhf * d.ring * kHeadDim, d.ring);
+                  reinterpret_cast<const __half*>(c.v_resid) + bhf * d.ring * kHeadDim, d.ring,
+                  X.img_p == (int)bhf ? image : nullptr);
             }
           }
           if (X.i1 > X.i0) {
@@ -1134,8 +1154,8 @@ size_t smem_bytes(const Dims& d) {
   const int page = (int)d.page_bytes;
   const size_t rings = (size_t)kWarps * warp_ring_bytes(page) +
                        (size_t)kWarps * ring_slots(page) * sizeof(uint64_t);
-  // + the zero rows of the zero-point MMAs
-  return (rings + kZeroBytes + 16 + 127) / 128 * 128;
+  // + a flushed block's image and the zero rows of the zero-point MMAs
+  return (rings + image_bytes(page) + kZeroBytes + 16 + 127) / 128 * 128;
 }
 
 template <int BK, int BV, bool kWide>
