@@ -217,6 +217,8 @@ __device__ __forceinline__ __half order_half(int k) {
 // unless neighbouring fp16 numbers share a d (t far smaller than lo: 6 groups
 // in 10000 of Gaussian data) or the group is not finite; that is seen by
 // testing t and a neighbour, and then false is returned.
+// A NaN among finite numbers takes code 1 (an unordered comparison), as the
+// bits of a NaN y in quantize_codes do.
 // A comparison gives a mask per half, so element 2p reaches its bit 2p
 // directly for p < 8 and element 2p + 1 for p >= 8; the others are collected
 // one half-word off: a comparison and two ANDs per pair, where the fused
@@ -234,7 +236,7 @@ __device__ __forceinline__ bool threshold_codes(const __half2 (&x)[kGroup / 2], 
   uint32_t here = 0u, off = 0u;
 #pragma unroll
   for (int p = 0; p < kGroup / 2; ++p) {
-    const uint32_t m = __hgt2_mask(x[p], t);
+    const uint32_t m = __hgtu2_mask(x[p], t);
     here |= m & (p < 8 ? 1u << (2 * p) : 2u << (2 * p));
     off |= m & (p < 8 ? 0x20000u << (2 * p) : 1u << (2 * p - 16));
   }

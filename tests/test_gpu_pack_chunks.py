@@ -52,3 +52,23 @@ def test_any_chunking_gives_the_same_cache(kvq_lib, bits, chunk, residual, paged
             assert torch.equal(one.head_pages(b, h, nb), many.head_pages(b, h, nb))
     for x, y in zip(_window(one, L), _window(many, L)):
         assert torch.equal(x, y)
+
+
+def test_one_bit_codes_of_nan(kvq_lib):
+    """A NaN among finite numbers gets the same 1-bit code in a long call (the
+    threshold) as in short ones (the definition's arithmetic): equal bytes."""
+    cfg = kvq.CacheConfig(batch=1, n_q_heads=2, n_kv_heads=2, bits_k=1, bits_v=1, max_len=256,
+                          residual=32)
+    g = torch.Generator().manual_seed(8)
+    k, v = (torch.randn(1, 2, 224, 128, generator=g).half() for _ in range(2))
+    for x in (k, v):
+        x[torch.rand(x.shape, generator=g) < 0.02] = float("nan")
+    pages = []
+    for step in (224, 7):
+        cache = kvq.QuantKVCache(cfg)
+        for i in range(0, 224, step):
+            kvq.kvq_pack(cache, k[:, :, i:i + step].contiguous().cuda(),
+                         v[:, :, i:i + step].contiguous().cuda())
+        torch.cuda.synchronize()
+        pages.append(cache.pages()[:, :, :6].cpu())
+    assert torch.equal(*pages)
