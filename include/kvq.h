@@ -240,7 +240,7 @@ int32_t kvq_attn_default_splits(const kvq_config* cfg);
  * device).  lengths: host int32 [batch], each in [0, max_len].
  *   kvq_attn_default_splits (the split plan) when one wave of its CTAs fills
  *   at least 90% of the GPU, as for batch-1 decoding, where a launch is
- *   bound by latency and dedicated window warps keep the fp16 chunks off the
+ *   bound by latency and dedicated window warps keep the fp16 window off the
  *   block warps' path; otherwise 0, the flat plan, which streams every pair
  *   in one wave (no CTA start and merges per wave).
  * Returns -1 on an invalid argument.
@@ -266,9 +266,9 @@ kvq_status kvq_workspace_init(void* workspace, size_t ws_bytes, void* stream);
  *   softmax_scale  0 selects 1/sqrt(128).
  *   n_splits       the work plan.  1..255: the split plan, n_splits CTAs per
  *                  (sequence, kv-head) pair share its 32-token blocks
- *                  (contiguous ranges, one per warp) and its window chunks
+ *                  (contiguous ranges, one per warp) and its window
  *                  (dedicated warps).  0: the flat plan, one CTA per SM; all
- *                  pairs' blocks and window chunks lie end to end, weighted
+ *                  pairs' blocks and window tokens lie end to end, weighted
  *                  by their measured cost, and every warp takes an equal
  *                  contiguous share, crossing pair boundaries as it goes.
  *                  Either way a pair's CTAs (and a warp that leaves a pair

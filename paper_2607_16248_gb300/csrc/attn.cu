@@ -1,16 +1,16 @@
 // kvq_decode_attn: one decode step of grouped-query attention
 // softmax(q K^T * scale) V (Sec. 1 of the paper) over the packed KbVb cache.
 //
-// Grid (S, n_kv_heads, batch) of 512-thread CTAs, one per SM.  The S CTAs
-// of one (sequence, kv-head) share its work: the packed 32-token blocks and
-// the 32-token chunks of the fp16 residual window are cut into contiguous
-// ranges, one per warp (a warp takes only blocks or only window chunks).
+// This file is the flat plan (n_splits = 0): one 512-thread CTA per SM.  The
+// packed 32-token blocks and the 16-token units of the fp16 residual window
+// of all (sequence, kv-head) pairs lie end to end, weighted by cost, and every
+// warp takes an equal contiguous range (see Costs); it may cross pairs.
 // Each warp streams its own pages into a private ring of shared-memory slots
 // with bulk asynchronous copies (cp.async.bulk + one mbarrier per slot) and
-// keeps a running softmax state.  The warps of a CTA merge in shared memory
-// into one partial (max, sum, unnormalised row) per query head; with S > 1
-// the last CTA of a (sequence, kv-head) to finish (atomic ticket, no
-// waiting) merges the S partials:
+// keeps a running softmax state.  The warps of a CTA that end in the same pair
+// merge in shared memory into one partial (max, sum, unnormalised row) per
+// query head; the last of a pair's partials to be written (atomic ticket, no
+// waiting) merges them:
 //   out = sum_s 2^{m_s - M} o_s / sum_s 2^{m_s - M} l_s.
 // Scores are kept in the log2 domain (scaled by softmax_scale * log2 e).
 //
@@ -544,7 +544,7 @@ __device__ __noinline__ TcState tc_window_units(TcState st, const Dims d, const 
 
 // Inverse of tc_write_state<false>: a WarpState (natural channel order) back
 // into registers in the window layout (channel = 16 m-tile + row, no
-// zero-point term), so the window chunks of a pair continue the state its
+// zero-point term), so the window units of a pair continue the state its
 // packed blocks began.  Row sums go to the lanes of gid 0.
 template <bool kWide>
 __device__ __forceinline__ void tc_read_state(TcState& st, const WarpState& ws, int lane) {
@@ -816,12 +816,16 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
         const int n = tc_pre_issue<BK, BV>(page_map(d, c, w.b, w.h), tw, j0, j1, s.nb - 1, ring,
                                            full, R, end, flag);
         // A block that leaves the window here: its rows are at least
-        // `residual` tokens old, so the first warp of the CTA that owns one
-        // quantizes it now into the CTA's image (used if the lengths hold).
+        // `residual` >= 32 tokens old, so the first warp of the CTA that owns
+        // one quantizes it now into the CTA's image (used if the lengths hold;
+        // then only the previous step's newest row, which it does not hold, can
+        // still be on its way).  The fence orders the rows behind the length:
+        // a long kvq_pack call may have written them just before it.
         if (w.L > w.L0 && s.Lq > packed_len(w.L0, d.residual) && j1 == s.nb && j1 > j0) {
           int taken = 1;
           if (lane == 0) taken = atomicExch(&image_taken, 1);
           if (__shfl_sync(0xffffffffu, taken, 0) == 0) {
+            __threadfence();
             const long long ro = ((long long)w.b * d.hkv + w.h) * d.ring * kHeadDim;
             for (int qi = 0; qi < 4; ++qi)
               flush_quarter<BK, BV>(reinterpret_cast<const __half*>(c.k_resid) + ro,

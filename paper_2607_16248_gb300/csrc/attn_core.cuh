@@ -273,7 +273,7 @@ struct TcState {
 //     row sum and in the value MMAs (so they are a consistent softmax of
 //     scores perturbed by at most 2^-11 relative); pt holds p~ (column =
 //     head; narrow: columns 4..7 zero), pl is unused.
-// kSumL: add the weights to st.l here (window chunks).  Packed blocks leave
+// kSumL: add the weights to st.l here (window units).  Packed blocks leave
 // it: their row sums come out of the value zero-point MMA, whose A row 4 is
 // all ones (see tc_unit).
 template <int NB, bool kWide, bool kCompact, bool kSumL>
@@ -694,14 +694,14 @@ __device__ __forceinline__ void tc_write_state(const TcState& st, WarpState& ws,
 // ---------------------------------------------------------------------------
 // Tensor-core path for the fp16 residual window (the flat plan, and the split
 // plan's short ranges, take 16-token units, further below): a warp stages the
-// K rows of a 32-token chunk in shared memory, scores them with ldmatrix-fed MMAs
+// K rows of a 32-token unit in shared memory, scores them with ldmatrix-fed MMAs
 // (keys as A with tokens as rows), then stages the V rows in the same place
 // (values transposed, channels as rows).  Rows past the window are zero and
 // their scores -inf.
 // ---------------------------------------------------------------------------
 
 constexpr int kResRow = kHeadDim + 8;                    // halves per staged row (16-byte pad)
-constexpr int kResRowsBytes = kGroup * kResRow * 2;      // one 32-row K or V chunk
+constexpr int kResRowsBytes = kGroup * kResRow * 2;      // the K or V rows of a 32-token unit
 
 __device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], const void* p) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
@@ -817,8 +817,8 @@ __host__ __device__ constexpr int ring_slots(int page) {
          : kRingBudget / (kWarps * ring_blocks(page) * page) > 4 ? 4
                                                                  : kRingBudget / (kWarps * ring_blocks(page) * page);
 }
-// A warp's ring: its slots, and at least one 32-row K (or V) chunk of the
-// window, which a window warp stages there.
+// A warp's ring: its slots, and at least the 32 K (or V) rows of a
+// 32-token window unit, which a window warp stages there.
 __host__ __device__ constexpr int warp_ring_bytes(int page) {
   return ((ring_slots(page) * ring_blocks(page) * page > kResRowsBytes
                ? ring_slots(page) * ring_blocks(page) * page

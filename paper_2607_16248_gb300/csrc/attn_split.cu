@@ -7,8 +7,8 @@
 //
 // Grid (S, n_kv_heads, batch) of 512-thread CTAs, one per SM.  The S CTAs
 // of one (sequence, kv-head) share its work: the packed 32-token blocks and
-// the 32-token chunks of the fp16 residual window are cut into contiguous
-// ranges, one per warp (a warp takes only blocks or only window chunks).
+// the 16- or 32-token units of the fp16 residual window (Plan) are cut into
+// contiguous ranges, one per warp (a warp takes only blocks or only units).
 // Each warp streams its own pages into a private ring of shared-memory slots
 // with bulk asynchronous copies (cp.async.bulk + one mbarrier per slot) and
 // keeps a running softmax state.  The warps of a CTA merge in shared memory

@@ -103,3 +103,41 @@ def test_steps_enqueued_back_to_back(kvq_lib, n_splits, paged):
     rms = b.square().mean(-1, keepdim=True).sqrt()
     # the two paths differ by fp32 summation order
     assert float(((a - b).abs() / rms).max()) <= 1e-4
+
+
+@pytest.mark.parametrize("bits", [1, 4])
+def test_flushing_step_behind_a_long_append(kvq_lib, bits):
+    """Every step flushes a block whose ring rows the append just before it
+    wrote (95 tokens, then one step, five times): the same lengths and
+    results with the calls enqueued back to back as with a wait after each."""
+    cfg = kvq.CacheConfig(batch=2, n_q_heads=8, n_kv_heads=2, bits_k=bits, bits_v=bits,
+                          max_len=512, residual=32)
+    kv = [synth.kv_heads(60 + b, 2, 480) for b in range(2)]
+    k, v = (torch.stack([kv[b][j] for b in range(2)]).cuda() for j in range(2))
+    q = torch.stack([synth.queries(70 + i, 2, 8) for i in range(5)]).cuda()
+    packs = [[x[:, :, 96 * i:96 * i + 95].contiguous() for x in (k, v)] for i in range(5)]
+    news = [[x[:, :, 96 * i + 95].contiguous() for x in (k, v)] for i in range(5)]
+    res = []
+    for wait in (False, True):
+        cache = kvq.QuantKVCache(cfg)
+        ws = kvq.attn_workspace(cfg, 0)
+        torch.cuda.synchronize()
+        outs = []
+        for i in range(5):
+            kvq.kvq_pack(cache, *packs[i])
+            if wait:
+                torch.cuda.synchronize()
+            outs.append(kvq.kvq_decode_step(cache, *news[i], q[i], n_splits=0, workspace=ws,
+                                            out_dtype=torch.float32))
+            if wait:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        assert cache.flags() == 0 and cache.seq_lens().tolist() == [480, 480]
+        # once more over all the blocks
+        outs.append(kvq.kvq_decode_attn(cache, q[0], n_splits=1, workspace=kvq.attn_workspace(cfg, 1),
+                                        out_dtype=torch.float32))
+        res.append(torch.stack(outs))
+    # partials merge in an order that may differ between runs: fp32 rounding
+    a, b = res
+    rms = b.square().mean(-1, keepdim=True).sqrt()
+    assert float(((a - b).abs() / rms).max()) <= 1e-5
