@@ -18,7 +18,8 @@
 // row that its guesses do not settle (thousands of nearly equal logits around
 // a boundary, alpha = 1) it leaves to the general kernel, launched behind it,
 // which takes any row with one cluster of 8 CTAs.  256 rows of 128256 on a
-// GB300: 1050 us with the general kernel alone, 160 with both.
+// GB300: 1050 us with the general kernel alone, 160 with both.  Launches of a
+// few long rows go to the general kernel alone (launch_drift).
 //
 // The general kernel.  Each CTA stages an eighth of both logit rows in shared
 // memory once (the only HBM read) and the CTAs combine their partial results
@@ -1003,6 +1004,8 @@ __device__ void drift_row(Sm& s, const float* __restrict__ z_fp, const float* __
   cluster_sync();  // no CTA goes on while a peer may read its shared memory
 }
 
+// kAll: every row, one cluster each (no streaming kernel ran).
+template <bool kAll>
 __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kT, 1)
     drift_general_kernel(const float* __restrict__ z_fp, const float* __restrict__ z_q, int rows,
                          int vocab, kvq_drift_params p, int32_t* __restrict__ m_t,
@@ -1012,6 +1015,10 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kT, 1)
   Sm& s = *reinterpret_cast<Sm*>(smem_raw);
   pdl_launch_dependents();
   pdl_wait();  // the streaming kernel's marks
+  if constexpr (kAll) {
+    drift_row(s, z_fp, z_q, blockIdx.y, vocab, p, m_t, c_t, d_loc, y_t, cov);
+    return;
+  }
   // Marks are read kT rows at a time (usually none is set).  Every CTA of the
   // cluster reads them before the barriers that come before rank 0 overwrites
   // one.
@@ -1023,9 +1030,10 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kT, 1)
     __shared__ uint32_t marks[kT / 32];
     if ((threadIdx.x & 31) == 0) marks[threadIdx.x >> 5] = bal;
     __syncthreads();
-    for (int k = 0; k < kT; ++k)
-      if (marks[k >> 5] >> (k & 31) & 1u)
-        drift_row(s, z_fp, z_q, r0 + k * (int)gridDim.y, vocab, p, m_t, c_t, d_loc, y_t, cov);
+    for (int w = 0; w < kT / 32; ++w)
+      for (uint32_t bits = marks[w]; bits; bits &= bits - 1u)
+        drift_row(s, z_fp, z_q, r0 + (32 * w + __ffs(bits) - 1) * (int)gridDim.y, vocab, p, m_t,
+                  c_t, d_loc, y_t, cov);
     __syncthreads();
   }
 }
@@ -1919,9 +1927,24 @@ cudaError_t launch_drift(const float* z_fp, const float* z_q, int rows, int voca
   int sms = 0;
   cudaError_t e = sm_count(&sms);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(drift_general_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sizeof(Sm));
+    e = cudaFuncSetAttribute(drift_general_kernel<false>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Sm));
   if (e != cudaSuccess) return e;
+  const int clusters = sms / kCl > 0 ? sms / kCl : 1;
+  // A few long rows: a cluster spreads each over eight SMs, and up to 15 run at
+  // once.  The line lies where a CTA's stream of a row takes as long, which
+  // falls with alpha (more of the row belongs to C): 7 rows, sigma 2.1 to 3.9,
+  // alpha 0.9: 32768: 32 to 36 us streamed, 36 to 40 in clusters; 49152: 36 to 44
+  // and 39 to 44; 98304: 51 to 63 and 47 to 54.  alpha 0.99: 24576: 30 to 38 and
+  // 36 to 40; 32768: 34 to 44 and 37 to 42; 98304: 56 to 81 and 50 to 59.
+  if (rows * 10 <= sms && vocab > (p.alpha > 0.97f ? 28672 : 40960)) {
+    e = cudaFuncSetAttribute(drift_general_kernel<true>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Sm));
+    if (e != cudaSuccess) return e;
+    drift_general_kernel<true><<<dim3(kCl, rows), kT, sizeof(Sm), st>>>(
+        z_fp, z_q, rows, vocab, p, m_t, c_t, d_loc, y_t, cov);
+    return cudaGetLastError();
+  }
   // at most one row per SM: all of an SM's threads on it
   e = rows <= sms ? launch_stream<1024>(z_fp, z_q, rows, vocab, p, m_t, c_t, d_loc, y_t, cov, st)
                   : launch_stream<512>(z_fp, z_q, rows, vocab, p, m_t, c_t, d_loc, y_t, cov, st);
@@ -1933,13 +1956,12 @@ cudaError_t launch_drift(const float* z_fp, const float* z_q, int rows, int voca
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const int clusters = sms / kCl > 0 ? sms / kCl : 1;
   cfg.gridDim = dim3(kCl, rows < clusters ? rows : clusters);
   cfg.blockDim = dim3(kT);
   cfg.dynamicSmemBytes = sizeof(Sm);
   cfg.stream = st;
-  return cudaLaunchKernelEx(&cfg, drift_general_kernel, z_fp, z_q, rows, vocab, p, m_t, c_t, d_loc,
-                            y_t, cov);
+  return cudaLaunchKernelEx(&cfg, drift_general_kernel<false>, z_fp, z_q, rows, vocab, p, m_t,
+                            c_t, d_loc, y_t, cov);
 }
 
 cudaError_t launch_drift_window(const float* cov, int rows, int k_max, float rho_k,

@@ -46,6 +46,22 @@ def test_row_counts(kvq_lib, rows):
     _compare(zf, zq, 0.8, 4, 12, 0.02, 0.5, rows=pick, require=0.6)
 
 
+@pytest.mark.parametrize("V", [40960, 40961, 131075, 163840])
+def test_few_long_rows(kvq_lib, V):
+    """Launches of few long rows go to the general kernel, longer ones (40
+    rows: on either side of the rule for any SM count) to the streaming one:
+    the same decisions and, the terms being the same integers, sums."""
+    zf, zq = (z.cuda() for z in synth.paired_logits(V, 40, V, sigma=2.5, noise=0.4))
+    whole = kvq.drift_metrics(zf, zq, 0.95, 8, 100, 0.02, 0.5)
+    for lo, n in ((0, 1), (1, 16), (17, 17)):
+        part = kvq.drift_metrics(zf[lo:lo + n], zq[lo:lo + n], 0.95, 8, 100, 0.02, 0.5)
+        for k in ("m_t", "y_t", "c_t", "cov"):
+            assert torch.equal(part[k], whole[k][lo:lo + n]), k
+        # its sums of products run in another order: double-float rounding
+        torch.testing.assert_close(part["d_loc"], whole["d_loc"][lo:lo + n], rtol=1e-6, atol=2e-7)
+    _compare(zf[:2].cpu(), zq[:2].cpu(), 0.95, 8, 100, 0.02, 0.5, require=0.6)
+
+
 @pytest.mark.parametrize("shift", [1, 2, 3])
 def test_unaligned_rows(kvq_lib, shift):
     # each array's rows start at 4-byte alignments of their own
