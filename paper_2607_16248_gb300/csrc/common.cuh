@@ -298,8 +298,29 @@ __device__ __forceinline__ uint32_t gather_nibbles(uint32_t row, int gid, Src sr
 // body quantizes both groups in turn (half the instructions to fetch).
 // Used by kvq_pack and by the decode step's flush, which are therefore
 // bit-identical.
-template <int BK, int BV, typename RowK, typename RowV>
-__device__ __forceinline__ void quantize_quarter(RowK row_k, RowV row_v, int qi, char* image) {
+// The loads: xk = tokens 2p, 2p + 1 of the lane's channel, xv = channels 2p,
+// 2p + 1 of its token.
+template <typename RowK, typename RowV>
+__device__ __forceinline__ void load_quarter(RowK row_k, RowV row_v, int qi,
+                                             __half2 (&xk)[kGroup / 2],
+                                             __half2 (&xv)[kGroup / 2]) {
+  const int lane = threadIdx.x & 31, c = kGroup * qi + lane;
+#pragma unroll
+  for (int p = 0; p < kGroup / 2; ++p) xk[p] = __halves2half2(row_k(2 * p)[c], row_k(2 * p + 1)[c]);
+  const uint4* row = reinterpret_cast<const uint4*>(row_v(lane) + kGroup * qi);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const uint4 u = row[k];
+    const uint32_t wd[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) xv[4 * k + e] = *reinterpret_cast<const __half2*>(&wd[e]);
+  }
+}
+
+template <int BK, int BV>
+__device__ __forceinline__ void quantize_loaded(__half2 (&xk)[kGroup / 2],
+                                                const __half2 (&xv)[kGroup / 2], int qi,
+                                                char* image) {
   const int lane = threadIdx.x & 31;
   const int gid = lane >> 2, tig = lane & 3;
   uint32_t* kcodes = reinterpret_cast<uint32_t*>(image);
@@ -308,19 +329,6 @@ __device__ __forceinline__ void quantize_quarter(RowK row_k, RowV row_v, int qi,
   __half* vmeta = reinterpret_cast<__half*>(image + page_off_vmeta(BK, BV));
   const int c = kGroup * qi + lane;  // this lane's key channel
   const int vm = vmeta_index(qi, lane);
-  __half2 xk[kGroup / 2], xv[kGroup / 2];  // tokens 2p, 2p + 1 / channels 2p, 2p + 1
-#pragma unroll
-  for (int p = 0; p < kGroup / 2; ++p) xk[p] = __halves2half2(row_k(2 * p)[c], row_k(2 * p + 1)[c]);
-  {
-    const uint4* row = reinterpret_cast<const uint4*>(row_v(lane) + kGroup * qi);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const uint4 u = row[k];
-      const uint32_t wd[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-      for (int e = 0; e < 4; ++e) xv[4 * k + e] = *reinterpret_cast<const __half2*>(&wd[e]);
-    }
-  }
   uint32_t rk = 0u, rv = 0u;  // 1-bit code rows
   if constexpr (BK == BV) {
 #pragma unroll 1
@@ -372,6 +380,13 @@ __device__ __forceinline__ void quantize_quarter(RowK row_k, RowV row_v, int qi,
     vcodes[4 * lane + qi] = gather_nibbles(
         rv, gid, [&](int k) { return 8 * tig + 4 * (k >> 2) + (k & 3); },
         [](int k) { return 10 + 16 * (k >> 2) - 4 * (k & 3); });
+}
+
+template <int BK, int BV, typename RowK, typename RowV>
+__device__ __forceinline__ void quantize_quarter(RowK row_k, RowV row_v, int qi, char* image) {
+  __half2 xk[kGroup / 2], xv[kGroup / 2];
+  load_quarter(row_k, row_v, qi, xk, xv);
+  quantize_loaded<BK, BV>(xk, xv, qi, image);
 }
 
 

@@ -173,16 +173,6 @@ __device__ __forceinline__ RowSrc make_src(const Dims& d, const kvq_cache& c, co
   return s;
 }
 
-// A block whose first tokens are in the ring (at most residual / 32 + 1 per
-// call and kv-head).  Out of line: the kernel's body stays the one of the
-// blocks made of new tokens only.
-template <int BK, int BV>
-__device__ __noinline__ void quantize_mixed_quarter(const RowSrc src, int j, int qi, char* page) {
-  quantize_quarter<BK, BV>(
-      [&](int t) { return reinterpret_cast<const __half*>(src.k(j * kGroup + t)); },
-      [&](int t) { return reinterpret_cast<const __half*>(src.v(j * kGroup + t)); }, qi, page);
-}
-
 // Every block that leaves the window in a call of more than 32 tokens: one
 // warp per quarter of a block (quantize_quarter: key channels 32 w .. 32 w +
 // 31 and value group w), reading the rows straight from the input (or the
@@ -191,11 +181,15 @@ __device__ __noinline__ void quantize_mixed_quarter(const RowSrc src, int j, int
 // append kernel behind this one.  grid (blocks, hkv, batch_count) of 128
 // threads.  (With the four or five blocks that begin in the ring left to the
 // append kernel, one after another in one CTA per kv-head, a 4099-token chunk
-// of 4 x 8 heads at 4 bits took 49 us; here they are CTAs like the others.)
+// of 4 x 8 heads at 4 bits took 49 us; here they are CTAs like the others.
+// Only their loads differ: with an out-of-line call for them the kernel took
+// 7 registers more, and 128k tokens, K4V2, 220 us against 202.)
 constexpr int kInputThreads = 4 * 32;
 
+// Equal widths: 64 or 56 registers, 8 or 9 CTAs per SM (K4V4 with one CTA
+// fewer 147 against 141 us); the others stay within 72 by themselves.
 template <int BK, int BV>
-__global__ void __launch_bounds__(kInputThreads)
+__global__ void __launch_bounds__(kInputThreads, BK != BV ? 1 : BK == 8 ? 8 : 9)
     pack_input_blocks_kernel(Dims d, kvq_cache c, const __half* __restrict__ k_new,
                              const __half* __restrict__ v_new, int n_new, int batch_begin) {
   pdl_enter();
@@ -207,17 +201,24 @@ __global__ void __launch_bounds__(kInputThreads)
   if (j >= packed_len(L1, d.residual) / kGroup) return;
   char* page = page_ptr(d, c, b, h, j);
   if (!page) return;
-  if (j * kGroup < L0) {
-    quantize_mixed_quarter<BK, BV>(make_src(d, c, k_new, v_new, n_new, b, bi, h, L0), j,
-                                   threadIdx.x >> 5, page);
-    return;
-  }
   const long long nh = ((long long)bi * d.hkv + h) * n_new;
   const __half* nk = k_new + (nh + (long long)j * kGroup - L0) * kHeadDim;
   const __half* nv = v_new + (nh + (long long)j * kGroup - L0) * kHeadDim;
-  quantize_quarter<BK, BV>([&](int t) { return nk + (long long)t * kHeadDim; },
-                           [&](int t) { return nv + (long long)t * kHeadDim; },
-                           threadIdx.x >> 5, page);
+  __half2 xk[kGroup / 2], xv[kGroup / 2];
+  const int n_ring = L0 - j * kGroup;  // tokens of the block that are in the ring
+  if (n_ring > 0) {
+    // the ring's length is a multiple of 32: a block's rows lie together
+    const long long ro = (((long long)b * d.hkv + h) * d.ring + (j * kGroup) % d.ring) * kHeadDim;
+    const __half* rk = reinterpret_cast<const __half*>(c.k_resid) + ro;
+    const __half* rv = reinterpret_cast<const __half*>(c.v_resid) + ro;
+    load_quarter([&](int t) { return (t < n_ring ? rk : nk) + (long long)t * kHeadDim; },
+                 [&](int t) { return (t < n_ring ? rv : nv) + (long long)t * kHeadDim; },
+                 threadIdx.x >> 5, xk, xv);
+  } else {
+    load_quarter([&](int t) { return nk + (long long)t * kHeadDim; },
+                 [&](int t) { return nv + (long long)t * kHeadDim; }, threadIdx.x >> 5, xk, xv);
+  }
+  quantize_loaded<BK, BV>(xk, xv, threadIdx.x >> 5, page);
 }
 
 template <int BK>
