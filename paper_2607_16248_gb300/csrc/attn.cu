@@ -124,15 +124,18 @@ struct MergeGroups {
 // ---------------------------------------------------------------------------
 
 // Cost weights: a window unit costs cw units, the first item of a pair sc
-// more (measured: about 2 to 4 blocks' time, a pair start ~1; with 1, 2 and
-// 4 units the ragged batch below took 372, 337 and 330 us for four layers, and
-// 8 x 64k K1V1 414, 386 and 385), and the
-// block that leaves the window in a decode step fu more (its warp quantizes
-// the block alone; Mistral-7B shape, K2V2, ragged batch of 16 where some
-// sequence flushes on most steps: 0, 4, 8 and 12 units gave 4.30, 4.24,
-// 4.19 and 4.18 ms mean and 4.70, 4.54, 4.40 and 4.37 ms p95 per 32-layer
-// step).  A launch with too little work
-// for every warp to hold an item under those weights takes lighter ones
+// more (about one block's time), and the block that leaves the window in a
+// decode step fu more (its warp quantizes the block alone; Mistral-7B shape,
+// K2V2, ragged batch of 16 where some sequence flushes on most steps: 0, 4, 8
+// and 12 units gave 4.30, 4.24, 4.19 and 4.18 ms mean and 4.70, 4.54, 4.40 and
+// 4.37 ms p95 per 32-layer step).  cw = 2, although a unit takes up to four
+// blocks' time: what the windows cost, the block ranges of all other warps
+// are longer by, and an fp32 accumulator's error grows with the blocks it
+// takes.  With 1, 2 and 4 units the ragged batch took 372, 333 and 331 us for
+// four layers and 8 x 64k K1V1 414, 389 and 386; the error of the ragged
+// batch's fp32 results against 64 bits is 8.6e-5 with 4 units and 8.4e-5
+// with 2 (one unit of 32 tokens at 4: 8.5e-5).  A launch with too little
+// work for every warp to hold an item under those weights takes lighter ones
 // (FlatGrid::k), down to one unit per item.
 struct Costs {
   int cw, sc, fu;
@@ -174,7 +177,7 @@ __host__ __device__ inline int items_below(long long x, int nb, int nr, Costs k,
   const int lo_w = nb == 0 ? 1 : 0;
   if (nr > lo_w) {
     const long long t = x - k.sc - nb - f;
-    const int sh = k.cw == 4 ? 2 : k.cw == 2 ? 1 : 0;  // cw is 1, 2 or 4
+    const int sh = k.cw >> 1;  // log2 of cw: 1, 2 or 4
     const long long n = t <= 0 ? 0 : (t + k.cw - 1) >> sh;
     c += (int)max(0LL, min(n, (long long)nr) - lo_w);
   }
@@ -218,7 +221,7 @@ __host__ __device__ inline FlatGrid flat_grid(const WorkSums& w, int ctas) {
   const long long cap = (long long)kWarps * ctas;
   // the heaviest weights under which every one of the cap warps can still
   // hold an item start (each range >= the largest item cost)
-  const Costs pick[3] = {{4, 1, 12}, {1, 1, 6}, {1, 0, 0}};
+  const Costs pick[3] = {{2, 1, 12}, {1, 1, 6}, {1, 0, 0}};
   int i = 0;
   for (; i < 2; ++i) {
     const long long N = w.nb + pick[i].cw * w.nr + pick[i].sc * w.np + pick[i].fu * w.nf;
