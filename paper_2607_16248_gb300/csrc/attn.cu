@@ -36,8 +36,8 @@
 //
 // Codes become fp16 values without a table: for 1-bit codes (stored in
 // fragment order) a rotated bit lands on an exponent bit (value 2^e), codes
-// of 2 bits (and 4 in the wide layout) are moved to the top of the mantissa of
-// a subnormal number, and wider ones are OR-ed into the mantissa of 1024 and
+// of 2 bits (and 4 in the wide layout) are moved to the top of the low eleven
+// bits of a number with no other bits (Codes, attn_core.cuh), and wider ones are OR-ed into the mantissa of 1024 and
 // 1024 is subtracted.  The resulting per-row power-of-two factors are undone on the
 // fp32 results.  The fp16 residual window takes the same MMAs with operands
 // loaded by ldmatrix from rows staged in shared memory.

@@ -133,31 +133,33 @@ __device__ __forceinline__ uint32_t hsub1024(uint32_t x) {
 // channels for keys, two tokens for values): v[j] = (f_j code_a, f_j code_b)
 // as fp16, exact.  inv(j) = 1 / f_j.
 //
-// Codes of 2 bits (and 4 in the wide layout) are taken as they lie in the ten
-// mantissa bits of an fp16 number whose exponent field is zero: bit i of it is
-// 2^(i - 24), so a code at bit i is code 2^i 2^-24, exactly, and an operand
-// register is one AND, where OR-ing the code into the mantissa of 1024 and
-// subtracting 1024 (the other widths) takes one instruction more: 128 of about
-// 600 for a K2V2 block.  The MMA aligns a product by its operands' exponent
-// fields, so a code k bits below the top of the mantissa loses k bits of the
-// accumulator's alignment.  Left at the bottom of the mantissa that costs 100
-// times the error; so each code is moved to the top bits, or two bits below
-// them where that saves a shift.  Error of fp32 results against 64 bits,
-// relative, mean over query groups of 1, 2, 4 and 5 and four seeds at 6000
-// tokens: K2V2 2.61e-6 with the subtraction, 2.60e-6 without; K4V4 in groups
-// of 5: 3.42e-6 and 3.05e-6, but in groups of up to 4 heads 2.52e-6 and
-// 2.71e-6, so the narrow layout keeps the subtraction for 4 bits.  Ragged
-// batch of 16 (8k to 32k tokens, 8 heads, groups of 4), K2V2: 109 -> 89 us.
+// Codes of 2 bits (and 4 in the wide layout) are taken as they lie in the low
+// eleven bits of an fp16 number: bit i is 2^(i - 24) for i <= 10 (the bits of
+// 0 .. 2^11 - 1 are the values 0 .. (2^11 - 1) 2^-24, subnormal or not), so a
+// code at bit i is code 2^i 2^-24, exactly, and an operand register is one
+// AND, where OR-ing the code into the mantissa of 1024 and subtracting 1024
+// (the other widths) takes one instruction more.  The MMA aligns a product by
+// its operands' exponent fields, and all subnormal numbers share one, so a
+// code k bits below bit 10 loses k bits of the accumulator's alignment.
+// (kVal) Value codes therefore end at bit 10, or two bits below for half of
+// the 2-bit ones; the accumulators they add to are often no larger than one
+// product.  Key codes, whose scores add up over 128 channels, keep the
+// positions that cost one multiplication for four registers.  Error of fp32
+// results against 64 bits, 400 to 20000 tokens, against the subtraction: K1V2
+// -11 to -24%, K1V4 in groups of 5 and 8 within 0.2%, K2V2 -4 to -12%, K2V4
+// within 3%; with value codes ending at bits 9 and 7, K1V2 was up to 36% and
+// K1V4 25% further off.  Ragged batch of 16 (8k to 32k tokens, 8 heads, groups
+// of 4), K2V2, per layer: 109 us with the subtraction, 90 without.
 constexpr float kSub = 16777216.0f;  // 2^24
-template <int B, bool kWide>
+template <int B, bool kWide, bool kVal>
 struct Codes;
 
 // 1-bit codes are stored in fragment order (key1_bit / val1_bit): the word
 // w of a lane rotated left by 4 r holds, at bit 10 + 16 e + j, the code of
 // row j and half e of one fragment register, so each register is one AND
 // (an fp16 with a single exponent bit set: 2^-14, 2^-13, 2^-11, 2^-7).
-template <bool kWide>
-struct Codes<1, kWide> {
+template <bool kWide, bool kVal>
+struct Codes<1, kWide, kVal> {
   __device__ static constexpr float inv(int j) {
     return j == 0 ? 16384.0f : j == 1 ? 8192.0f : j == 2 ? 2048.0f : 128.0f;
   }
@@ -176,7 +178,7 @@ __device__ __forceinline__ uint32_t comp(const uint4& u, int i) {
   return i == 0 ? u.x : i == 1 ? u.y : i == 2 ? u.z : u.w;
 }
 template <bool kWide>
-struct Codes<2, kWide> {
+struct Codes<2, kWide, false> {
   __device__ static constexpr float inv(int j) {
     return j == 0 || j == 2 ? kSub / 256.0f : kSub / 64.0f;
   }
@@ -190,8 +192,23 @@ struct Codes<2, kWide> {
     v[3] = x & 0x00C000C0u;
   }
 };
-template <>
-struct Codes<4, false> {
+template <bool kWide>
+struct Codes<2, kWide, true> {
+  __device__ static constexpr float inv(int j) {
+    return j == 0 || j == 2 ? kSub / 512.0f : kSub / 128.0f;
+  }
+  __device__ static int word(int gid) { return gid >> 2; }
+  __device__ static void get(uint32_t a, uint32_t b, uint32_t sel, uint32_t (&v)[4]) {
+    const uint32_t x = __byte_perm(a, b, sel);  // the lane's byte -> both bytes of each half
+    const uint32_t y = x * 2u, z = x * 32u;
+    v[0] = y & 0x06000600u;
+    v[1] = z & 0x01800180u;
+    v[2] = z & 0x06000600u;
+    v[3] = y & 0x01800180u;
+  }
+};
+template <bool kVal>
+struct Codes<4, false, kVal> {
   __device__ static constexpr float inv(int j) { return (j & 1) ? 0.0625f : 1.0f; }
   __device__ static int word(int gid) { return gid >> 1; }
   __device__ static void get(uint32_t a, uint32_t b, uint32_t sel, uint32_t (&v)[4]) {
@@ -204,7 +221,7 @@ struct Codes<4, false> {
   }
 };
 template <>
-struct Codes<4, true> {
+struct Codes<4, true, false> {
   __device__ static constexpr float inv(int j) { return (j & 1) ? kSub / 16.0f : kSub / 64.0f; }
   __device__ static int word(int gid) { return gid >> 1; }
   __device__ static void get(uint32_t a, uint32_t b, uint32_t sel, uint32_t (&v)[4]) {
@@ -216,8 +233,21 @@ struct Codes<4, true> {
     v[3] = y & 0x00F000F0u;
   }
 };
-template <bool kWide>
-struct Codes<8, kWide> {
+template <>
+struct Codes<4, true, true> {
+  __device__ static constexpr float inv(int) { return kSub / 128.0f; }
+  __device__ static int word(int gid) { return gid >> 1; }
+  __device__ static void get(uint32_t a, uint32_t b, uint32_t sel, uint32_t (&v)[4]) {
+    const uint32_t x = __byte_perm(a, b, sel);            // the lane's 16 bits -> each half
+    const uint32_t y = __byte_perm(a, b, sel ^ 0x1111u);  // their bytes swapped
+    v[0] = (x * 128u) & 0x07800780u;
+    v[1] = (x * 8u) & 0x07800780u;
+    v[2] = (y * 128u) & 0x07800780u;
+    v[3] = (y * 8u) & 0x07800780u;
+  }
+};
+template <bool kWide, bool kVal>
+struct Codes<8, kWide, kVal> {
   __device__ static constexpr float inv(int) { return 1.0f; }
   __device__ static int word(int gid) { return gid; }
   __device__ static void get(uint32_t a, uint32_t b, uint32_t, uint32_t (&v)[4]) {
@@ -409,11 +439,11 @@ __device__ __forceinline__ void tc_unit(const char* const (&pg)[NB], const char*
       for (int half = 0; half < 2; ++half) {
         uint32_t v[4];
         if constexpr (BK == 1) {
-          Codes<1, kWide>::rot(comp(kw1[bi], ks >> 1), 2 * (ks & 1) + half, v);
+          Codes<1, kWide, false>::rot(comp(kw1[bi], ks >> 1), 2 * (ks & 1) + half, v);
         } else {
           const uint32_t wa = *reinterpret_cast<const uint32_t*>(kc + 4 * ((c + 2 * half) * BK + ln.wk));
           const uint32_t wb = *reinterpret_cast<const uint32_t*>(kc + 4 * ((c + 2 * half + 1) * BK + ln.wk));
-          Codes<BK, kWide>::get(wa, wb, ln.sel_k, v);
+          Codes<BK, kWide, false>::get(wa, wb, ln.sel_k, v);
         }
         a0[2 * half] = v[0];
         a0[2 * half + 1] = v[1];
@@ -471,7 +501,7 @@ __device__ __forceinline__ void tc_unit(const char* const (&pg)[NB], const char*
           const int j = 2 * mt + rh;
           const float d = dk[bi][mt][2 * rh + hh];
           const float full = kWide ? d : d + __shfl_xor_sync(0xffffffffu, d, 2);
-          sc[bi][j][hh] = fmaf(full, Codes<BK, kWide>::inv(j) * scale_log2, hh ? z1 : z0);
+          sc[bi][j][hh] = fmaf(full, Codes<BK, kWide, false>::inv(j) * scale_log2, hh ? z1 : z0);
         }
   }
 
@@ -508,7 +538,7 @@ __device__ __forceinline__ void tc_unit(const char* const (&pg)[NB], const char*
           for (int dl = 0; dl < 2; ++dl) {
             const int ia = 2 * ks + dl;
             uint32_t v[4];
-            Codes<1, kWide>::rot(comp(vw, g), ia, v);
+            Codes<1, kWide, true>::rot(comp(vw, g), ia, v);
             am0[2 * dl] = v[0];
             am0[2 * dl + 1] = v[1];
             am1[2 * dl] = v[2];
@@ -567,8 +597,8 @@ __device__ __forceinline__ void tc_unit(const char* const (&pg)[NB], const char*
         for (int dl = 0; dl < 2; ++dl) {
           const int ia = 2 * ks + dl, ib = ia + 4;  // tokens 8tig + ia, 8tig + ib
           uint32_t v[4];
-          if constexpr (BV == 1) Codes<1, kWide>::rot(comp(vw1, g), ia, v);
-          else Codes<BV, kWide>::get(cw[ia], cw[ib], ln.sel_v, v);
+          if constexpr (BV == 1) Codes<1, kWide, true>::rot(comp(vw1, g), ia, v);
+          else Codes<BV, kWide, true>::get(cw[ia], cw[ib], ln.sel_v, v);
           am0[2 * dl] = v[0];
           am0[2 * dl + 1] = v[1];
           am1[2 * dl] = v[2];
@@ -603,8 +633,8 @@ __device__ __forceinline__ Lane make_lane(int lane) {
   ln.tig = lane & 3;
   ln.sel_k = code_selector<BK>(ln.gid);
   ln.sel_v = code_selector<BV>(ln.gid);
-  ln.wk = Codes<BK, false>::word(ln.gid);
-  ln.wv = Codes<BV, false>::word(ln.gid);
+  ln.wk = Codes<BK, false, false>::word(ln.gid);
+  ln.wv = Codes<BV, false, true>::word(ln.gid);
   ln.neg_lo = ln.gid >= 4 ? 0xBC00BC00u : 0u;
   ln.p_lo = ln.tig >= 2 ? 1.0f : 0.0f;
   return ln;
@@ -678,7 +708,7 @@ __device__ __forceinline__ void tc_write_state(const TcState& st, WarpState& ws,
       for (int rh = 0; rh < 2; ++rh) {
         const int jp = 2 * half + rh;
         const int cch = kPacked ? 32 * g + 4 * gid + jp : 16 * mtp + gid + 8 * rh;
-        const float inv = kPacked ? Codes<BV, kWide>::inv(jp) : 1.0f;
+        const float inv = kPacked ? Codes<BV, kWide, true>::inv(jp) : 1.0f;
 #pragma unroll
         for (int hh = 0; hh < 2; ++hh) {
           const float a = st.acc[mtp][2 * rh + hh];
