@@ -1837,13 +1837,14 @@ __global__ void __launch_bounds__(kS, 1024 / kS)
 constexpr int kWinT = 1024;
 constexpr int kWinLoads = 16;
 __global__ void __launch_bounds__(kWinT)
-    drift_window_kernel(const float* __restrict__ cov, int rows, int k_max, float rho_k,
+    drift_window_kernel(const float* cov, int rows, int k_max, float rho_k,
                         float* __restrict__ mean_cov, int32_t* __restrict__ k_b) {
   __shared__ double part[kWinT];
   __shared__ double col[kMaxKcov];
   __shared__ int best[kMaxKcov / 32];
   const int t = threadIdx.x, rank = (int)blockIdx.x, ctas = (int)gridDim.x;  // one cluster
-  pdl_wait();
+  pdl_wait();  // this kernel may start while cov is still being written: the loads
+               // below are coherent ones (not __ldg, nor through a restrict pointer)
   const int per = kWinT / k_max;  // rows per sweep of a CTA
   const int step = per * ctas;
   Cs sum;
@@ -1853,7 +1854,7 @@ __global__ void __launch_bounds__(kWinT)
       float v[kWinLoads];
 #pragma unroll
       for (int i = 0; i < kWinLoads; ++i)
-        v[i] = r + i * step < rows ? __ldg(cov + (r + i * step) * k_max + k) : 0.0f;
+        v[i] = r + i * step < rows ? __ldcg(cov + (r + i * step) * k_max + k) : 0.0f;
 #pragma unroll
       for (int i = 0; i < kWinLoads; ++i) sum.add(v[i]);
     }
