@@ -470,8 +470,7 @@ kvq_status kvq_drift_metrics(const float* z_fp, const float* z_q, int32_t rows,
  * kvq_drift_window — K_b of Sec. 4.1: the smallest k whose coverage
  * cov[.][k-1], averaged over the rows, reaches rho_k; 0 if none does.
  *   cov       device fp32 [rows][k_max] (from kvq_drift_metrics).
- *   mean_cov  device fp32 [k_max]: the column means (compensated fp32 sums of
- *             each thread's rows, good to 2^-46, added in fp64 in a fixed
+ *   mean_cov  device fp32 [k_max]: the column means (fp64 sums, in a fixed
  *             order).
  *   k_b       device int32 [1].
  */

@@ -1827,15 +1827,25 @@ __global__ void __launch_bounds__(kS, 1024 / kS)
 }
 
 // K_b: column means of cov over the rows and the smallest k whose mean reaches
-// rho_K (0 if none).  One CTA, or a cluster of 8 for more than 64
-// rows of every thread: a thread takes one column of every (CTAs kWinT /
-// k_max)-th row, sixteen loads in flight, and the partial sums are added in a
-// fixed order in fp64 (rows of a CTA, then CTAs).  A thread's own rows add up
-// in a compensated fp32 sum, good to 2^-46: fp64 additions and conversions run
-// at two a cycle and SM here (256 rows of 256: 43 us in one CTA with them, 11
-// in eight, and 41 when each thread walked all rows of a column).
+// rho_K (0 if none).  One CTA, or a cluster of 8 for more than kWinRows rows
+// of every thread: a thread takes one column of every (CTAs kWinT / k_max)-th
+// row, sixteen loads in flight, and adds its rows up in fp64; the partial sums
+// are added in a fixed order (pairwise in a CTA, then CTAs).  K_b compares these
+// means with rho_K, so they keep fp64's precision throughout (a pair of floats
+// whose low word is not renormalised loses 6 to 9 bits of it over 512 to 2048
+// rows).  What bounds it is fp64: two additions a cycle and SM, and conversions
+// slower by far (24 rows of 64: 12.0 us with them, 4.9 with widen).
 constexpr int kWinT = 1024;
 constexpr int kWinLoads = 16;
+constexpr int kWinRows = 8;  // 4 rows a thread: 7.1 us in one CTA and in eight; 16: 13.8 and 7.1
+// A float as a double, by integer steps where it is a normal number.
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t u = __float_as_uint(x);
+  if ((u & 0x7f800000u) - 0x00800000u < 0x7f000000u)
+    return __hiloint2double((int)(((u >> 3) & 0x0fffffffu) + 0x38000000u | (u & 0x80000000u)),
+                            (int)(u << 29));
+  return (double)x;
+}
 __global__ void __launch_bounds__(kWinT)
     drift_window_kernel(const float* cov, int rows, int k_max, float rho_k,
                         float* __restrict__ mean_cov, int32_t* __restrict__ k_b) {
@@ -1847,8 +1857,8 @@ __global__ void __launch_bounds__(kWinT)
                // below are coherent ones (not __ldg, nor through a restrict pointer)
   const int per = kWinT / k_max;  // rows per sweep of a CTA
   const int step = per * ctas;
-  Cs sum;
   if (t < per * k_max) {
+    double sum = 0.0;
     const int k = t % k_max;
     for (long long r = rank * per + t / k_max; r < rows; r += kWinLoads * step) {
       float v[kWinLoads];
@@ -1856,16 +1866,19 @@ __global__ void __launch_bounds__(kWinT)
       for (int i = 0; i < kWinLoads; ++i)
         v[i] = r + i * step < rows ? __ldcg(cov + (r + i * step) * k_max + k) : 0.0f;
 #pragma unroll
-      for (int i = 0; i < kWinLoads; ++i) sum.add(v[i]);
+      for (int i = 0; i < kWinLoads; ++i)
+        if (r + i * step < rows) sum += widen(v[i]);
     }
-    part[t] = (double)sum.hi + (double)sum.lo;
+    part[t] = sum;
   }
   __syncthreads();
-  if (t < k_max) {
-    double c = 0.0;
-    for (int i = 0; i < per; ++i) c += part[i * k_max + t];
-    col[t] = c;
+  for (int n = min(per, rows); n > 1;) {  // the threads of a column, pairwise
+    const int h = (n + 1) / 2;
+    if (t < (n - h) * k_max) part[t] += part[t + h * k_max];
+    __syncthreads();
+    n = h;
   }
+  if (t < k_max) col[t] = part[t];
   cluster_sync();  // (one CTA: a block barrier)
   int mine = 0x7fffffff;
   if (rank == 0 && t < kMaxKcov) {
@@ -1968,7 +1981,7 @@ cudaError_t launch_drift(const float* z_fp, const float* z_q, int rows, int voca
 cudaError_t launch_drift_window(const float* cov, int rows, int k_max, float rho_k,
                                 float* mean_cov, int32_t* k_b, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
-  const int ctas = (long long)rows * k_max > 64 * kWinT ? kCl : 1;
+  const int ctas = (long long)rows * k_max > kWinRows * kWinT ? kCl : 1;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
