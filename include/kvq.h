@@ -457,8 +457,9 @@ int32_t kvq_drift_max_vocab(void);
  *   m_t        device int32 [rows]; c_t, d_loc device fp32 [rows];
  *   y_t        device uint8 [rows]; cov device fp32 [rows][k_max].
  * Probabilities are e^(z - max z) in fp32; masses are summed as multiples of
- * 2^-40, products in double-float, and combined in fp64 (c_t, d_loc are the
- * fp64 results rounded to fp32).  rows <= 65535, vocab <= 163840.
+ * 2^-40, products as multiples of 2^-60, and combined in fp64 (c_t, d_loc are
+ * the fp64 results rounded to fp32): a row's results depend on nothing but the
+ * row, and repeat bit for bit.  rows <= 65535, vocab <= 163840.
  * No workspace; calls on different outputs may overlap.
  */
 kvq_status kvq_drift_metrics(const float* z_fp, const float* z_q, int32_t rows,

@@ -35,12 +35,13 @@
 //      index order);
 //   3. the same selection by count on z_q gives the k_max-th element, then
 //      the k_max best elements are gathered and sorted (the TopK order);
-//   4. one pass over U: its masses (fixed point) and the sums of e_fp^2,
-//      e_fp e_q, e_q^2 (double-float), from which d_loc follows.
+//   4. one pass over U: its masses and the sums of e_fp^2, e_fp e_q, e_q^2
+//      (multiples of 2^-60), from which d_loc follows.
 // A mass term e = expf(z - m) (fp32, in (0, 1]) is taken as an integer
 // multiple of 2^-40 (round to nearest) and every mass sum is an exact 64-bit
-// integer sum: the same numbers decide every comparison, in any order, and
-// no per-element fp64 arithmetic is needed.
+// integer sum, the product sums likewise (Prod): the same numbers decide every
+// comparison, in any order, no per-element fp64 arithmetic is needed, and a row
+// has the same results in either kernel, in every run and beside any rows.
 
 #include <float.h>
 
@@ -79,7 +80,7 @@ struct Sm {
   uint32_t rc[kBins / kCl];
   u64 rm[kBins / kCl];
   u64 xin[kCl][kXw];                // values loaded from the eight CTAs
-  u64 xin8[kCl][2 * kXw];           // the same for a two-slot exchange
+  u64 xin3[kCl][3 * kXw];           // the same for the three slots of a row's sums
   u64 wsel[kMaxKcov];               // coverage terms of the TopK list
   float bc[4];                      // broadcast scalars
   uint32_t ru[kW];
@@ -152,38 +153,49 @@ __device__ __forceinline__ u64 fix40(float e) {
 }
 constexpr double kFix = 1099511627776.0;  // 2^40
 
-// Double-float accumulator: an unevaluated sum hi + lo of two floats
-// (error-free transformations: two-sum and the fma product residual).
-struct Df {
-  float hi = 0.0f, lo = 0.0f;
-  __device__ __forceinline__ void add(float x) {
-    const float s = hi + x;
-    const float bb = s - hi;
-    const float e = (hi - (s - bb)) + (x - bb);
-    const float l = lo + e;
-    hi = s + l;
-    lo = l - (hi - s);
+// A sum of products of terms in [0, 1] as whole multiples of 2^-60, so that
+// neither the order nor the split of the additions can change it (at most
+// 2047 products a thread).  A product is p + r exactly; adding 8 rounds p to a
+// multiple of 2^-20, adding 1.5 2^-17 rounds what is left of p, and r, to
+// multiples of 2^-40, and 1.5 2^-37 the last rest to one of 2^-60.  The
+// largest term of either row is 1 and belongs to U, so the sums of squares are
+// at least 1.
+struct Prod {
+  uint32_t hi = 0u, mid = 0u, low = 0u;  // in units of 2^-20, 2^-40 and 2^-60
+  __device__ __forceinline__ void add(float a, float b) {
+    constexpr float kMid = 1.5f / 131072.0f, kLow = 1.5f / 137438953472.0f;
+    constexpr uint32_t kMidBits = 0x37400000u, kLowBits = 0x2d400000u;
+    const float p = __fmul_rn(a, b), r = __fmaf_rn(a, b, -p);
+    const float h = __fadd_rn(p, 8.0f);
+    const float p1 = __fsub_rn(p, __fsub_rn(h, 8.0f));
+    const float m = __fadd_rn(p1, kMid), n = __fadd_rn(r, kMid);
+    const float p2 = __fsub_rn(p1, __fsub_rn(m, kMid)), r2 = __fsub_rn(r, __fsub_rn(n, kMid));
+    hi += __float_as_uint(h) - 0x41000000u;
+    mid += (__float_as_uint(m) - kMidBits) + (__float_as_uint(n) - kMidBits);
+    low += __float_as_uint(__fadd_rn(__fadd_rn(p2, r2), kLow)) - kLowBits;
   }
-  __device__ __forceinline__ void add(const Df& o) {
-    add(o.hi);
-    add(o.lo);
+  __device__ __forceinline__ u64 coarse() const {  // multiples of 2^-40
+    return ((u64)hi << 20) + (u64)(long long)(int)mid;
   }
-  __device__ __forceinline__ void add_prod(float a, float b) {
-    const float p = a * b;
-    add(p);
-    add(fmaf(a, b, -p));
-  }
-  __device__ __forceinline__ u64 pack() const {
-    return ((u64)__float_as_uint(hi) << 32) | __float_as_uint(lo);
-  }
-  __device__ static Df unpack(u64 w) {
-    Df d;
-    d.hi = __uint_as_float((uint32_t)(w >> 32));
-    d.lo = __uint_as_float((uint32_t)w);
-    return d;
-  }
-  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+  __device__ __forceinline__ u64 fine() const { return (u64)(long long)(int)low; }
 };
+__device__ __forceinline__ double prod_value(u64 coarse, u64 fine) {
+  return ((double)(long long)coarse + (double)(long long)fine / 1048576.0) / kFix;
+}
+// The words of a row's sums over U, all whole numbers: count, masses A, B and C
+// (see write_row), then coarse and fine parts of the sums of e_fp^2, e_fp e_q
+// and e_q^2.
+constexpr int kSumWords = 10;
+__device__ __forceinline__ void warp_sums(u64 (&w)[kSumWords], u64* out) {  // by lane 0
+#pragma unroll
+  for (int o = 16; o; o >>= 1)
+#pragma unroll
+    for (int k = 0; k < kSumWords; ++k) w[k] += __shfl_xor_sync(0xffffffffu, w[k], o);
+  if ((threadIdx.x & 31) == 0) {
+#pragma unroll
+    for (int k = 0; k < kSumWords; ++k) out[k] = w[k];
+  }
+}
 
 // (key, index) packed so that a larger word ranks first: key descending,
 // index ascending.
@@ -269,23 +281,6 @@ __device__ void cluster_gather(Sm& s, int slot, u64 a, u64 b, u64 c = 0ull, u64 
   if (threadIdx.x < kXw * kCl)
     s.xin[threadIdx.x / kXw][threadIdx.x % kXw] =
         ld_peer_u64(peer_addr(&s.xd[slot][threadIdx.x % kXw], threadIdx.x / kXw));
-  __syncthreads();
-}
-// Six words in slots `slot` and `slot + 1`, one barrier; s.xin8[rank][word].
-__device__ void cluster_gather2x(Sm& s, int slot, u64 a, u64 b, u64 c, u64 d, u64 e, u64 f) {
-  if (threadIdx.x == 0) {
-    s.xd[slot][0] = a;
-    s.xd[slot][1] = b;
-    s.xd[slot][2] = c;
-    s.xd[slot][3] = d;
-    s.xd[slot + 1][0] = e;
-    s.xd[slot + 1][1] = f;
-  }
-  cluster_sync();
-  if (threadIdx.x < 2 * kXw * kCl) {
-    const int r = threadIdx.x / (2 * kXw), w = threadIdx.x % (2 * kXw);
-    s.xin8[r][w] = ld_peer_u64(peer_addr(&s.xd[slot + w / kXw][w % kXw], (uint32_t)r));
-  }
   __syncthreads();
 }
 __device__ __forceinline__ void cluster_gather2(Sm& s, int slot, u64 a, u64 b) {
@@ -752,15 +747,16 @@ __device__ __forceinline__ bool ranks_in(uint32_t k, uint32_t i, const Pick& p) 
   return p.all || k > p.key || (k == p.key && i <= p.idx);
 }
 
-// Row results from the masses A = e_fp(U), B = e_q(U), c_sum = e_fp(C and S),
-// S_fp and the product sums (one thread).
-__device__ void write_row(int row, int32_t len, u64 A, u64 B, u64 c_sum, double sf, const Df& saa,
-                          const Df& sab, const Df& sbb, const kvq_drift_params& p, int32_t* m_t,
-                          float* c_t, float* d_loc, uint8_t* y_t) {
-  const double ia = kFix / (double)A, ib = kFix / (double)B;
-  double dsum = saa.value() * ia * ia - 2.0 * sab.value() * ia * ib + sbb.value() * ib * ib;
+// Row results from S_fp and the sums over U (kSumWords of them): masses A =
+// e_fp(U), B = e_q(U), C = e_fp(C and S) and the product sums (one thread).
+__device__ void write_row(int row, int32_t len, const u64* w, double sf, const kvq_drift_params& p,
+                          int32_t* m_t, float* c_t, float* d_loc, uint8_t* y_t) {
+  const double ia = kFix / (double)w[1], ib = kFix / (double)w[2];
+  const double saa = prod_value(w[4], w[5]), sab = prod_value(w[6], w[7]),
+               sbb = prod_value(w[8], w[9]);
+  double dsum = saa * ia * ia - 2.0 * sab * ia * ib + sbb * ib * ib;
   if (dsum < 0.0) dsum = 0.0;  // rounding of an exact zero
-  const double c = (double)c_sum / sf;
+  const double c = (double)w[3] / sf;
   const double d = sqrt(dsum);
   m_t[row] = len;
   c_t[row] = (float)c;
@@ -868,14 +864,14 @@ __device__ void drift_row(Sm& s, const float* __restrict__ z_fp, const float* __
   __syncthreads();
 
   // ---- one pass over U = C union S ----
-  // masses A = e_fp(U), B = e_q(U), c = e_fp(C and S) in fixed point; the
-  // sums of e_fp^2, e_fp e_q, e_q^2 in double-float for
+  // masses A = e_fp(U), B = e_q(U), c = e_fp(C and S) and the sums of e_fp^2,
+  // e_fp e_q, e_q^2 (Prod) for
   //   d_loc^2 = Saa / A^2 - 2 Sab / (A B) + Sbb / B^2.
   // U is sparse: each warp queues its members (local index, bit 31 = in C
   // and S) in its own 64 entries of buf past the TopK list and works on them
   // 32 at a time, so the exponentials and products run on full warps.
   u64 A = 0ull, B = 0ull, Cs = 0ull;
-  Df saa, sab, sbb;
+  Prod saa, sab, sbb;
   {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     uint32_t* uq = reinterpret_cast<uint32_t*>(&s.buf[kMaxKcov]) + warp * 64;
@@ -886,9 +882,9 @@ __device__ void drift_row(Sm& s, const float* __restrict__ z_fp, const float* __
       A += qa;
       B += fix40(b);
       if (e >> 31) Cs += qa;
-      saa.add_prod(a, a);
-      sab.add_prod(a, b);
-      sbb.add_prod(b, b);
+      saa.add(a, a);
+      sab.add(a, b);
+      sbb.add(b, b);
     };
     int qn = 0;
     for (int t0 = warp * 32; t0 < cx.n; t0 += kT) {
@@ -914,77 +910,39 @@ __device__ void drift_row(Sm& s, const float* __restrict__ z_fp, const float* __
     }
     if (lane < qn) member(uq[lane]);
   }
-  // per-warp sums (a fixed pairing order), then thread 0 adds the warps
+  // the sums of the warps, of the CTA and, after one exchange, of the cluster
+  // (the count is the prefix length already)
   {
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-      A += __shfl_xor_sync(0xffffffffu, A, o);
-      B += __shfl_xor_sync(0xffffffffu, B, o);
-      Cs += __shfl_xor_sync(0xffffffffu, Cs, o);
-      Df* acc[3] = {&saa, &sab, &sbb};
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        Df w;
-        w.hi = __shfl_xor_sync(0xffffffffu, acc[k]->hi, o);
-        w.lo = __shfl_xor_sync(0xffffffffu, acc[k]->lo, o);
-        if ((threadIdx.x & o) == 0) {
-          acc[k]->add(w);
-        } else {
-          w.add(*acc[k]);
-          *acc[k] = w;
-        }
-      }
+    u64 w[kSumWords] = {0ull,          A,          B,            Cs,         saa.coarse(),
+                        saa.fine(), sab.coarse(), sab.fine(), sbb.coarse(), sbb.fine()};
+    u64* wpart = reinterpret_cast<u64*>(s.wsel);  // [kW][kSumWords] (wsel is free until the outputs)
+    warp_sums(w, wpart + (threadIdx.x >> 5) * kSumWords);
+    __syncthreads();
+    if (threadIdx.x < kSumWords) {
+      u64 v = 0ull;
+      for (int k = 0; k < kW; ++k) v += wpart[k * kSumWords + threadIdx.x];
+      s.xd[slot + threadIdx.x / kXw][threadIdx.x % kXw] = v;
     }
-    u64* wpart = reinterpret_cast<u64*>(s.wsel);  // [kW][6] (wsel is free until the outputs)
-    if ((threadIdx.x & 31) == 0) {
-      u64* w = wpart + (threadIdx.x >> 5) * 6;
-      w[0] = A;
-      w[1] = B;
-      w[2] = Cs;
-      w[3] = saa.pack();
-      w[4] = sab.pack();
-      w[5] = sbb.pack();
+    cluster_sync();
+    if (threadIdx.x < kSumWords * kCl) {
+      const uint32_t k = threadIdx.x % kSumWords, r = threadIdx.x / kSumWords;
+      s.xin3[r][k] = ld_peer_u64(peer_addr(&s.xd[slot + k / kXw][k % kXw], r));
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-      A = B = Cs = 0ull;
-      Df ta, tb, tc;
-      for (int w = 0; w < kW; ++w) {
-        A += wpart[w * 6];
-        B += wpart[w * 6 + 1];
-        Cs += wpart[w * 6 + 2];
-        ta.add(Df::unpack(wpart[w * 6 + 3]));
-        tb.add(Df::unpack(wpart[w * 6 + 4]));
-        tc.add(Df::unpack(wpart[w * 6 + 5]));
-      }
-      saa = ta;
-      sab = tb;
-      sbb = tc;
+    if (threadIdx.x < kSumWords) {
+      u64 v = 0ull;
+      for (int r = 0; r < kCl; ++r) v += s.xin3[r][threadIdx.x];
+      s.xin3[0][threadIdx.x] = v;
     }
     __syncthreads();
-  }
-  // one exchange of the six CTA totals (thread 0's values are published)
-  cluster_gather2x(s, slot, A, B, Cs, saa.pack(), sab.pack(), sbb.pack());
-  slot += 2;
-  u64 c_sum = 0ull;
-  if (threadIdx.x == 0) {
-    A = B = 0ull;
-    saa = sab = sbb = Df();
-    for (int r = 0; r < kCl; ++r) {
-      A += s.xin8[r][0];
-      B += s.xin8[r][1];
-      c_sum += s.xin8[r][2];
-      saa.add(Df::unpack(s.xin8[r][3]));
-      sab.add(Df::unpack(s.xin8[r][4]));
-      sbb.add(Df::unpack(s.xin8[r][5]));
-    }
+    slot += 3;
   }
 
   // ---- outputs (rank 0) ----
   if (cx.rank == 0) {
     if (threadIdx.x == 0)
-      write_row(row, pf.all ? vocab : (int32_t)pf.len, A, B, c_sum, (double)sf, saa, sab,
-                sbb, p, m_t, c_t, d_loc, y_t);
+      write_row(row, pf.all ? vocab : (int32_t)pf.len, s.xin3[0], (double)sf, p, m_t, c_t, d_loc,
+                y_t);
     // coverage curve: prefix sums of p_fp over TopK(z_q, k) within C; the
     // FP16 logits of the list come from the CTAs that hold them
     const int sl = ((vocab + kCl - 1) / kCl + 3) & ~3;
@@ -1103,7 +1061,7 @@ struct Ss {
     u64 set[kS];                  // finish: the elements around the boundary
   };
   u64 wsel[kMaxKcov];             // coverage terms
-  u64 part[kSw][8];               // warps' sums: count, A, B, C and S, saa, sab, sbb
+  u64 part[kSw][kSumWords];       // warps' sums
   u64 su[kSw], sv[kSw];
   float rf[4][kSw];
   uint32_t sc[2][kSw];
@@ -1186,26 +1144,6 @@ __device__ __forceinline__ float bin_floor(float a) {
   return (a - (float)(kBins - 1)) * (1.0f / kDepthScale);
 }
 
-// Compensated sum: hi + lo, lo collecting the rounding errors of hi.
-struct Cs {
-  float hi = 0.0f, lo = 0.0f;
-  __device__ __forceinline__ void add(float x, float rest = 0.0f) {
-    const float s = hi + x;
-    const float b = s - hi;
-    lo += ((hi - (s - b)) + (x - b)) + rest;
-    hi = s;
-  }
-  __device__ __forceinline__ void add_prod(float a, float b) {
-    const float p = a * b;
-    add(p, fmaf(a, b, -p));
-  }
-  __device__ __forceinline__ Df df() const {
-    Df d;
-    d.add(hi);
-    d.add(lo);
-    return d;
-  }
-};
 // A sum of terms e in [0, 1] as multiples of 2^-40 (fix40's value, at most
 // 4095 terms): e + 8 rounds e to a multiple of 2^-20, the exact rest + 1.5
 // 2^-17 to one of 2^-40.
@@ -1225,49 +1163,19 @@ struct Sums {
   uint32_t cnt = 0u;
   Fixed A, B;
   u64 C = 0ull;
-  Cs aa, ab, bb;
+  Prod aa, ab, bb;
   __device__ __forceinline__ void add(float a, float b) {
     A.add(a);
     B.add(b);
-    aa.add_prod(a, a);
-    ab.add_prod(a, b);
-    bb.add_prod(b, b);
+    aa.add(a, a);
+    ab.add(a, b);
+    bb.add(b, b);
   }
 };
-__device__ __forceinline__ void df_xor(Df& v, int o) {  // a fixed pairing order
-  Df w;
-  w.hi = __shfl_xor_sync(0xffffffffu, v.hi, o);
-  w.lo = __shfl_xor_sync(0xffffffffu, v.lo, o);
-  const bool up = (threadIdx.x & o) != 0;
-  const Df a = up ? w : v, b = up ? v : w;
-  v = a;
-  v.add(b);
-}
-// Sums over the warp into words out[0..6], by lane 0.
-__device__ __forceinline__ void warp_sums(u64 n, u64 A, u64 B, u64 C, Df aa, Df ab, Df bb,
-                                          u64* out) {
-#pragma unroll
-  for (int o = 16; o; o >>= 1) {
-    n += __shfl_xor_sync(0xffffffffu, n, o);
-    A += __shfl_xor_sync(0xffffffffu, A, o);
-    B += __shfl_xor_sync(0xffffffffu, B, o);
-    C += __shfl_xor_sync(0xffffffffu, C, o);
-    df_xor(aa, o);
-    df_xor(ab, o);
-    df_xor(bb, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    out[0] = n;
-    out[1] = A;
-    out[2] = B;
-    out[3] = C;
-    out[4] = aa.pack();
-    out[5] = ab.pack();
-    out[6] = bb.pack();
-  }
-}
 __device__ __forceinline__ void warp_sums(const Sums& v, u64* out) {
-  warp_sums(v.cnt, v.A.value(), v.B.value(), v.C, v.aa.df(), v.ab.df(), v.bb.df(), out);
+  u64 w[kSumWords] = {v.cnt,       v.A.value(),   v.B.value(), v.C,           v.aa.coarse(),
+                      v.aa.fine(), v.ab.coarse(), v.ab.fine(), v.bb.coarse(), v.bb.fine()};
+  warp_sums(w, out);
 }
 
 // Exclusive prefix of x over the threads; *total the sum.  buf: one word per
@@ -1802,25 +1710,13 @@ __global__ void __launch_bounds__(kS, 1024 / kS)
   warp_sums(sums, s.part[warp]);
   __syncthreads();
   if (warp == 0) {
-    u64 cnt = 0ull, A = 0ull, B = 0ull, C = 0ull;
-    Df aa, ab, bb;
-    if (lane < kSw) {
-      const u64* w = s.part[lane];
-      cnt = w[0];
-      A = w[1];
-      B = w[2];
-      C = w[3];
-      aa = Df::unpack(w[4]);
-      ab = Df::unpack(w[5]);
-      bb = Df::unpack(w[6]);
-    }
+    u64 w[kSumWords];
+#pragma unroll
+    for (int k = 0; k < kSumWords; ++k) w[k] = lane < kSw ? s.part[lane][k] : 0ull;
     __syncwarp();
-    warp_sums(cnt, A, B, C, aa, ab, bb, s.part[0]);
-    if (lane == 0) {
-      const u64* w = s.part[0];
-      write_row(row, (int32_t)w[0], w[1], w[2], w[3], sf, Df::unpack(w[4]), Df::unpack(w[5]),
-                Df::unpack(w[6]), p, m_t, c_t, d_loc, y_t);
-    }
+    warp_sums(w, s.part[0]);
+    if (lane == 0)
+      write_row(row, (int32_t)s.part[0][0], s.part[0], sf, p, m_t, c_t, d_loc, y_t);
   } else if (warp == 1) {
     write_curve(s.wsel, sf, row, p.k_max, cov);
   }
