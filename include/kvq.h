@@ -277,6 +277,13 @@ kvq_status kvq_workspace_init(void* workspace, size_t ws_bytes, void* stream);
  *                  a single partial is written directly.
  *   workspace      device, >= kvq_attn_workspace_bytes(cfg, n_splits), zeroed
  *                  once by kvq_workspace_init.
+ * The kernel is launched with programmatic stream serialization.  A kernel of
+ * the caller's ahead of it on the stream that lets its dependents start early
+ * (griddepcontrol.launch_dependents) may go on writing anything this call
+ * reads when n_splits is 0: before its dependency wait the flat plan uses the
+ * lengths alone, and looks at them again behind it.  With n_splits > 0 such a
+ * kernel must not write block_table or pages after that point: the split plan
+ * streams the first packed blocks ahead of the wait.
  * A sequence with L = 0 gets a zero output.  Calls that share a workspace
  * must not overlap on the GPU.
  */

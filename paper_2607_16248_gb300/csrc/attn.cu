@@ -367,9 +367,7 @@ __device__ __forceinline__ void walk_next(Walk& w, const int* seq_len, const Dim
 // Fold packed blocks [lo, hi) of one pair into st, streaming their pages
 // through the warp's ring.  *pos_io counts the ring slots the warp has used
 // in this kernel (slot pos % R, phase parity (pos / R) & 1) and moves past
-// this call's slots; `pre` slots holding blocks [lo_h, pre_end) were
-// streamed early from position 0 and are consumed without use unless this
-// range begins with them.  keep_tail: the block after hi leaves the window
+// this call's slots.  keep_tail: the block after hi leaves the window
 // in this kernel and folds after this call (tc_fold_flush); blocks fold in
 // units of NB from lo, as kvq_decode_attn folds lo .. hi after kvq_pack, so
 // if the range ends in a unit of one, that unit is not folded here and its
@@ -377,9 +375,9 @@ __device__ __forceinline__ void walk_next(Walk& w, const int* seq_len, const Dim
 // flushed block: both paths then take the same softmax updates (1-bit values
 // round their fp16 weights against the running maximum).
 template <int BK, int BV, bool kWide>
-__device__ __forceinline__ TcState tc_packed_warp(TcState st, const PageMap pm, int lo_h, int pre,
-                                                  int pre_end, int lo, int hi, char* ring,
-                                                  uint64_t* full, int* pos_io, const char* zero,
+__device__ __forceinline__ TcState tc_packed_warp(TcState st, const PageMap pm, int lo, int hi,
+                                                  char* ring, uint64_t* full, int* pos_io,
+                                                  const char* zero,
                                                   const __half* qh, int gq, float scale_log2,
                                                   unsigned* flag, bool keep_tail,
                                                   const char** tail_out) {
@@ -389,23 +387,19 @@ __device__ __forceinline__ TcState tc_packed_warp(TcState st, const PageMap pm, 
   constexpr int NB = ring_blocks(page);
   constexpr int R = ring_slots(page);
   const int lane = threadIdx.x & 31;
-  const bool reuse = pre > 0 && lo == lo_h && min(lo + pre * NB, hi) == pre_end;
-  const int skip = reuse ? 0 : pre;
-  const int n_units = hi > lo ? (hi - lo + NB - 1) / NB : 0;
-  const int total = skip + n_units;
+  const int total = hi > lo ? (hi - lo + NB - 1) / NB : 0;
   const int p0 = *pos_io;
-  const bool hold = keep_tail && NB == 2 && n_units > 0 && ((hi - lo) & 1);
+  const bool hold = keep_tail && NB == 2 && total > 0 && ((hi - lo) & 1);
   const char* tail = nullptr;
-  int issued = pre;  // slots issued so far
+  int issued = 0;  // slots issued so far
   auto real_issue = [&](int s) {
-    const int u = s - skip;
     // the slot may have been read (or written by generic stores: window rows,
     // a flushed page) before: order that before the copy that overwrites it
-    issue_slot<BK, BV>(pm, tw, ring, full, R, p0 + s, lo + u * NB, min(NB, hi - lo - u * NB), flag,
+    issue_slot<BK, BV>(pm, tw, ring, full, R, p0 + s, lo + s * NB, min(NB, hi - lo - s * NB), flag,
                        true);
     issued = s + 1;
   };
-  for (int s = pre; s < min(total, R); ++s) real_issue(s);
+  for (int s = 0; s < min(total, R); ++s) real_issue(s);
 
   const Lane ln = make_lane<BK, BV>(lane);
   uint32_t qb[16];
@@ -419,26 +413,23 @@ __device__ __forceinline__ TcState tc_packed_warp(TcState st, const PageMap pm, 
       break;
     }
     consumed = s + 1;
-    if (s >= skip) {
-      const int u = s - skip;
-      const char* base = ring + (size_t)slot * NB * page;
-      if (hold && s == total - 1) {
-        tail = base;
-      } else if (lo + u * NB + NB <= hi) {
-        const char* pg[NB];
+    const char* base = ring + (size_t)slot * NB * page;
+    if (hold && s == total - 1) {
+      tail = base;
+    } else if (lo + s * NB + NB <= hi) {
+      const char* pg[NB];
 #pragma unroll
-        for (int i = 0; i < NB; ++i) pg[i] = base + i * page;
-        tc_unit<BK, BV, NB, kWide>(pg, zero, qb, ln, scale_log2, st);
-      } else {
-        const char* pg[1] = {base};
-        tc_unit<BK, BV, 1, kWide>(pg, zero, qb, ln, scale_log2, st);
-      }
+      for (int i = 0; i < NB; ++i) pg[i] = base + i * page;
+      tc_unit<BK, BV, NB, kWide>(pg, zero, qb, ln, scale_log2, st);
+    } else {
+      const char* pg[1] = {base};
+      tc_unit<BK, BV, 1, kWide>(pg, zero, qb, ln, scale_log2, st);
     }
     __syncwarp();
     if (s + R < total) real_issue(s + R);
   }
-  // Copies issued but not consumed (a wait gave up, or the range shrank) land
-  // before the ring is reused; bounded waits.
+  // Copies issued but not consumed (a wait gave up) land before the ring is
+  // reused; bounded waits.
   if (lane == 0)
     for (int s = max(consumed, issued - R); s < issued; ++s)
       mbar_wait(full + (p0 + s) % R, ((p0 + s) / R) & 1);
@@ -451,27 +442,20 @@ __device__ __forceinline__ TcState tc_packed_warp(TcState st, const PageMap pm, 
 // The block `blk` of a pair leaves the window in this kernel (decode step)
 // and has no page yet: the warp quantizes it from the fp16 ring rows exactly
 // as kvq_pack does (quantize_quarter, common.cuh) into its idle ring (or the
-// second page of the held tail unit), unless that was done before the
-// dependency wait (`ready`: the image), writes the page and folds it, with the
+// second page of the held tail unit), writes the page and folds it, with the
 // tail unit if there is one.  Rare (one block in 32 steps), so out of line.
 template <int BK, int BV, bool kWide>
 __device__ __noinline__ TcState tc_fold_flush(TcState st, const PageMap pm, int blk,
                                               const char* tail, char* ring, const char* zero,
                                               const __half* qh, int gq, float scale_log2,
                                               unsigned* flag, const __half* ring_k,
-                                              const __half* ring_v, int ring_len,
-                                              char* ready) {
+                                              const __half* ring_v, int ring_len) {
   constexpr int page = page_bytes_c(BK, BV);
   const int lane = threadIdx.x & 31;
   TableWin tw;
   table_win_init(tw);
-  char* img = tail ? const_cast<char*>(tail) + page : ready ? ready : ring;
-  if (!ready) {
-    for (int qi = 0; qi < 4; ++qi) flush_quarter<BK, BV>(ring_k, ring_v, blk * kGroup, ring_len, qi, img);
-  } else if (img != ready) {  // beside the tail page
-    for (int i = lane; i < page / 16; i += 32)
-      reinterpret_cast<uint4*>(img)[i] = reinterpret_cast<const uint4*>(ready)[i];
-  }
+  char* img = tail ? const_cast<char*>(tail) + page : ring;
+  for (int qi = 0; qi < 4; ++qi) flush_quarter<BK, BV>(ring_k, ring_v, blk * kGroup, ring_len, qi, img);
   __syncwarp();
   char* dst = const_cast<char*>(block_addr(pm, tw, blk));
   if (dst) {
@@ -506,6 +490,19 @@ __device__ __forceinline__ void prefetch_rows_l2(const __half* ring_base, int p0
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(ring_base),
                  "r"((uint32_t)((n - n1) * kHeadDim * 2))
                  : "memory");
+}
+
+// Bring the pages of blocks [j0, j1) into L2 (a hint: nothing is taken from the
+// block table or the pages but the addresses, and a table entry is read past
+// L1, so that a later read sees the table as it is then).
+__device__ __forceinline__ void prefetch_pages_l2(const PageMap& pm, int j0, int j1) {
+  const int lane = threadIdx.x & 31;
+  for (int j = j0 + lane; j < (pm.paged() ? j1 : j0 + 1); j += 32) {
+    const char* src = pm.at(j, pm.paged() ? __ldcg(pm.row + j) : 0);
+    const uint32_t bytes = (uint32_t)((pm.paged() ? 1 : j1 - j0) * pm.page);
+    if (src)
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
+  }
 }
 
 // Window units [i0, i1) of one pair (unit u = tokens Lq + 16 u ...), K and V
@@ -699,9 +696,7 @@ struct WarpCtx {
   long long a, e;                // the warp's unit range
   int i0, i1;                    // the segment's window units
   int last, last_v;              // the segment ends the range; last virtual warp
-  int pre, pre_end, lo_h, p_h;   // early copies: count, end block, first block, pair
   int pos;                       // ring slots used
-  int img_p;                     // pair whose flushed block this warp holds as an image, or -1
   uint32_t wphase;               // window staging barrier parity count
   int j1;                        // the segment's end block
 };
@@ -721,7 +716,6 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
   __shared__ SegRec rec[kWarps];                  // each warp's final state (p < 0: none)
   __shared__ SegRec fin[kFinCap];                 // pairs whose partials this CTA completed
   __shared__ int fin_n;
-  __shared__ int image_taken;                     // the CTA's image of a flushed block is in use
   __shared__ int pub_last;
   __shared__ WarpCtx wctx[kWarps];                // each warp's walk and segment
   __shared__ FlatGrid grid_s;                     // the plan's grid
@@ -745,8 +739,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
   for (int i = threadIdx.x; i < kZeroBytes / 4; i += kThreads)
     zero[i] = i >= kOnesWord0 && i < kOnesWord0 + 16 ? 0x3C003C00u : 0u;
   unsigned* flag = reinterpret_cast<unsigned*>(c.seq_len) + d.batch;
-  if (threadIdx.x == 0) fin_n = image_taken = 0;
-  char* image = reinterpret_cast<char*>(smem + smem_size - 16 - kZeroBytes - image_bytes(page));
+  if (threadIdx.x == 0) fin_n = 0;
   if (lane == 0) {
     for (int i = 0; i < R; ++i) mbar_init(full + i, 1);
     mbar_init(&wbar[warp], 1);
@@ -757,12 +750,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 
   WarpCtx& X = wctx[warp];
   if (lane == 0) {
-    X.pre = 0;
-    X.pre_end = 0;
-    X.lo_h = -1;
-    X.p_h = -1;
     X.pos = 0;
-    X.img_p = -1;
     X.wphase = 0u;
     X.last = 0;
   }
@@ -794,14 +782,14 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
     }
   };
   // Before the dependency wait: the plan for the lengths as they are now, and
-  // the warp's first slots of blocks that no kernel still writes (a page never
-  // changes once written; the newest block of each pair may be the one the
-  // previous kernel is writing).  The lengths are compared after the wait, and
-  // the plan is made again if one changed (early slots that its range does not
-  // begin with are consumed without use).  A CTA starts here when the previous
-  // kernel's CTA on its SM has left and then waits for the slowest of that
-  // kernel's (7 to 14 us in a chain of layers), so this hides the plan (2.3 to
-  // 3 us) and the first copies (about 1.5 us).
+  // hints that bring the warp's first pages, and the ring rows of a block that
+  // leaves the window, into L2.  No other input is used before the wait: a
+  // kernel of the caller's that lets this one start early may still be writing
+  // the block table, the pages or the rings.  The lengths are compared after
+  // the wait, and the plan is made again if one changed.  A CTA starts here
+  // when the previous kernel's CTA on its SM has left and then waits for the
+  // slowest of that kernel's (7 to 14 us in a chain of layers), so this hides
+  // the plan (2.3 to 3 us) and most of the latency of the first copies.
   if (short_batch) {
     for (int b = threadIdx.x; b < d.batch; b += kThreads) len_s[b] = read_len(c.seq_len + b);
     __syncthreads();  // (and the zero rows are written)
@@ -813,37 +801,17 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
         const PairShape s = pair_shape(w.L, d.residual);
         const int j0 = min(items_below(X.a - U, s.nb, s.nr, g.k, w.f), s.nb);
         const int j1 = min(items_below(X.e - U, s.nb, s.nr, g.k, w.f), s.nb);
-        TableWin tw;
-        table_win_init(tw);
-        int end = 0;
-        const int n = tc_pre_issue<BK, BV>(page_map(d, c, w.b, w.h), tw, j0, j1, s.nb - 1, ring,
-                                           full, R, end, flag);
-        // A block that leaves the window here: its rows are at least
-        // `residual` >= 32 tokens old, so the first warp of the CTA that owns
-        // one quantizes it now into the CTA's image (used if the lengths hold;
-        // then only the previous step's newest row, which it does not hold, can
-        // still be on its way).  The fence orders the rows behind the length:
-        // a long kvq_pack call may have written them just before it.
-        if (w.L > w.L0 && s.Lq > packed_len(w.L0, d.residual) && j1 == s.nb && j1 > j0) {
-          int taken = 1;
-          if (lane == 0) taken = atomicExch(&image_taken, 1);
-          if (__shfl_sync(0xffffffffu, taken, 0) == 0) {
-            __threadfence();
-            const long long ro = ((long long)w.b * d.hkv + w.h) * d.ring * kHeadDim;
-            for (int qi = 0; qi < 4; ++qi)
-              flush_quarter<BK, BV>(reinterpret_cast<const __half*>(c.k_resid) + ro,
-                                    reinterpret_cast<const __half*>(c.v_resid) + ro,
-                                    s.Lq - kGroup, d.ring, qi, image);
-            if (lane == 0) X.img_p = w.b * d.hkv + w.h;
-          }
+        // (max_blocks: a length not yet initialised gives no address outside)
+        prefetch_pages_l2(page_map(d, c, w.b, w.h), j0,
+                          min(min(j1, j0 + R * ring_blocks(page)), d.max_blocks));
+        if (lane == 0 && w.L > w.L0 && s.Lq > packed_len(w.L0, d.residual) && j1 == s.nb &&
+            j1 > j0) {
+          const long long ro = ((long long)w.b * d.hkv + w.h) * d.ring * kHeadDim;
+          prefetch_rows_l2(reinterpret_cast<const __half*>(c.k_resid) + ro, s.Lq - kGroup, kGroup,
+                           d.ring);
+          prefetch_rows_l2(reinterpret_cast<const __half*>(c.v_resid) + ro, s.Lq - kGroup, kGroup,
+                           d.ring);
         }
-        if (lane == 0) {
-          X.pre = n;
-          X.pre_end = end;
-          X.lo_h = j0;
-          X.p_h = w.b * d.hkv + w.h;
-        }
-        __syncwarp();
       }
     }
   }
@@ -851,32 +819,16 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
   pdl_wait();
   bool stale = !short_batch;
   if (short_batch) {
-    for (int b = threadIdx.x; b < d.batch; b += kThreads) stale |= read_len(c.seq_len + b) != len_s[b];
+    for (int b = threadIdx.x; b < d.batch; b += kThreads) {
+      const int L0 = read_len(c.seq_len + b);
+      stale |= L0 != len_s[b];
+      len_s[b] = L0;
+    }
     stale = __syncthreads_or(stale);
   }
-  if (stale) {
-    if (lane == 0) X.img_p = -1;
-    if (short_batch) {
-      for (int b = threadIdx.x; b < d.batch; b += kThreads) len_s[b] = read_len(c.seq_len + b);
-      __syncthreads();
-    }
-    make_plan();
-  }
+  if (stale) make_plan();
   if (g.N == 0 && blockIdx.x == 0 && warp == 0)
     for (int i = lane; i < P * gq * kHeadDim; i += 32) store_out(out, out_f16, i, 0.0f);
-  // Early copies still in flight that no packed range consumed land before
-  // the ring is used otherwise (bounded waits).
-  auto drain_pre = [&]() {
-    const int pre = X.pre;
-    if (pre > 0) {
-      if (lane == 0) {
-        for (int s = 0; s < pre; ++s) mbar_wait(full + s % R, (s / R) & 1);
-        X.pos = pre;
-        X.pre = 0;
-      }
-      __syncwarp();
-    }
-  };
   // A state the warp leaves for the next pair: its pair's only partial goes
   // out directly, any other to the warp slot and the pair's ticket.
   auto emit_warp_partial = [&](const TcState& st, bool packed_kind, const SegRec& r,
@@ -975,18 +927,15 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
         TcState st;
         init_state(st);
         if (j1 > j0) {
-          // the early slots (ring positions 0 .. pre - 1) are this range's
-          // first ones if it begins where the early plan's did; a block that
-          // leaves the window in this kernel folds after the streamed ones
+          // a block that leaves the window in this kernel folds after the
+          // streamed ones
           const bool flush = grew && s.Lq > packed_len(w.L0, d.residual) && j1 == s.nb;
           const char* tail = nullptr;
-          st = tc_packed_warp<BK, BV, kWide>(st, page_map(d, c, w.b, w.h), p == X.p_h ? X.lo_h : -1,
-                                             X.pre, X.pre_end, j0, flush ? j1 - 1 : j1, ring, full,
-                                             &X.pos, reinterpret_cast<const char*>(zero),
+          st = tc_packed_warp<BK, BV, kWide>(st, page_map(d, c, w.b, w.h), j0, flush ? j1 - 1 : j1,
+                                             ring, full, &X.pos,
+                                             reinterpret_cast<const char*>(zero),
                                              q + head0 * kHeadDim, gq, scale_log2, flag, flush,
                                              &tail);
-          __syncwarp();
-          if (lane == 0) X.pre = 0;
           __syncwarp();
           {
             // the flush (segment read back from X)
@@ -999,8 +948,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
                   reinterpret_cast<const char*>(zero),
                   q + ((long long)wf.b * d.hq + (long long)wf.h * gq) * kHeadDim, gq, scale_log2,
                   flag, reinterpret_cast<const __half*>(c.k_resid) + bhf * d.ring * kHeadDim,
-                  reinterpret_cast<const __half*>(c.v_resid) + bhf * d.ring * kHeadDim, d.ring,
-                  X.img_p == (int)bhf ? image : nullptr);
+                  reinterpret_cast<const __half*>(c.v_resid) + bhf * d.ring * kHeadDim, d.ring);
             }
           }
           if (X.i1 > X.i0) {
@@ -1017,7 +965,6 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
         const Walk wr = X.w;
         const bool has_w = X.i1 > X.i0;
         if (has_w) {
-          drain_pre();
           const long long bh2 = (long long)wr.b * d.hkv + wr.h;
           const PairShape s2 = pair_shape(wr.L, d.residual);
           const bool grew2 = wr.L > wr.L0;
@@ -1028,7 +975,6 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
               scale_log2, grew2 ? wr.L0 : -1, grew2 ? k_new + bh2 * kHeadDim : nullptr,
               grew2 ? v_new + bh2 * kHeadDim : nullptr, &wbar[warp], &X.wphase, flag);
         }
-        drain_pre();
         if (X.last) {
           WarpState& t = *reinterpret_cast<WarpState*>(ring);
           if (!has_w) tc_write_state<true, BV, kWide>(st, t, lane);
@@ -1050,7 +996,6 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
       }
     }
   }
-  drain_pre();
   __syncthreads();
 
   // ---- merge the warps of this CTA that end in the same pair ----
@@ -1161,8 +1106,8 @@ size_t smem_bytes(const Dims& d) {
   const int page = (int)d.page_bytes;
   const size_t rings = (size_t)kWarps * warp_ring_bytes(page) +
                        (size_t)kWarps * ring_slots(page) * sizeof(uint64_t);
-  // + a flushed block's image and the zero rows of the zero-point MMAs
-  return (rings + image_bytes(page) + kZeroBytes + 16 + 127) / 128 * 128;
+  // + the zero rows of the zero-point MMAs
+  return (rings + kZeroBytes + 16 + 127) / 128 * 128;
 }
 
 template <int BK, int BV, bool kWide>
