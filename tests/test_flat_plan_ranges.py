@@ -26,7 +26,7 @@ int main() {
       chunks += (long long)hkv * ((L - s.Lq + 31) / 32);
     }
     const FlatGrid g = flat_grid(w, 152);
-    if (g.k.fu != 12) continue;  // lighter weights: little work
+    if (g.k.cw != 2) continue;  // lighter weights: little work
     // the range of a plan in which 32 window tokens cost four blocks
     const long long range = (w.nb + 4 * chunks + g.k.sc * w.np + g.n_v - 1) / g.n_v;
     CHECK((g.N + g.n_v - 1) / g.n_v <= range);
