@@ -999,6 +999,11 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
       }
     }
   }
+  // The warp that may publish the lengths puts what the kernels before this one
+  // wrote ahead of them (the split plan takes pages, but for the newest, by a
+  // length that it reads ahead of its dependency wait); here, where it waits
+  // for the others, the fence costs nothing (0.25 us at the publication).
+  if (append && warp == kWarps - 1) __threadfence();
   __syncthreads();
 
   // ---- merge the warps of this CTA that end in the same pair ----
@@ -1088,14 +1093,14 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
   __syncthreads();
 
   // ---- the decode step publishes the new lengths once every CTA is here ----
-  // (none reads a length after its ticket)
-  if (append && pub_last) {
-    for (int b = threadIdx.x; b < d.batch; b += kThreads) {
+  // (none reads a length after its ticket; by the warp that has fenced)
+  if (append && pub_last && warp == kWarps - 1) {
+    for (int b = lane; b < d.batch; b += 32) {
       const int L0 = read_len(c.seq_len + b);
-      if (L0 < d.max_len) c.seq_len[b] = L0 + 1;
+      if (L0 < d.max_len) *reinterpret_cast<volatile int*>(c.seq_len + b) = L0 + 1;
       else atomicOr(flag, (unsigned)KVQ_FLAG_OVERFLOW);
     }
-    if (threadIdx.x == 0) ws.tk[P] = 0u;
+    if (lane == 0) ws.tk[P] = 0u;
   }
 
   // ---- final merges of the pairs whose last partial came from this CTA ----

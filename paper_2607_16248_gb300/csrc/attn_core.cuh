@@ -95,6 +95,14 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ int read_len(const int* p) {
   return *reinterpret_cast<const volatile int*>(p);
 }
+// A length whose pages are read next, ahead of the dependency wait: what was
+// written before the length was published is seen behind this load (a fence
+// behind a plain load instead took 0.5 us a launch).
+__device__ __forceinline__ int read_len_acquire(const int* p) {
+  int n;
+  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(n) : "l"(p) : "memory");
+  return n;
+}
 
 __device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2,
                                          uint32_t a3, uint32_t b0, uint32_t b1) {
@@ -860,11 +868,11 @@ static_assert(kWarps * warp_ring_bytes(page_bytes_c(4, 8)) <= kRingBudget + 8 * 
 
 // Packed warps stream their blocks through a private ring of slots.  A page
 // is written once, when its group leaves the window, and never changes
-// afterwards, so before waiting for the previous kernel (programmatic
-// dependent launch) lane 0 already streams the first slots of the range that
-// a length read before the wait gives (tc_pre_issue), up to the block before
-// the newest.  If the range after the wait does not begin with exactly those
-// slots they are consumed without use.
+// afterwards, so in the split plan, before waiting for the previous kernel
+// (programmatic dependent launch), lane 0 already streams the first slots of
+// the range that a length read before the wait gives (tc_pre_issue), up to the
+// block before the newest.  If the range after the wait does not begin with
+// exactly those slots they are consumed without use.
 // A warp's window of 32 consecutive block-table entries (paged caches): lane
 // i holds the entry of block wb + i, refreshed (one coalesced load) when a
 // lookup leaves it.  Lookups are warp-uniform and made by all lanes.

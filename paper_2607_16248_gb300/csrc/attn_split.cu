@@ -145,8 +145,6 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 
 // Fold blocks [lo, hi) into st; `pre` slots holding blocks [lo_h, pre_end)
 // were streamed early.
-// Fold blocks [lo, hi) into st; `pre` slots holding blocks [lo_h, pre_end)
-// were streamed early.
 template <int BK, int BV, bool kWide>
 __device__ void tc_packed_warp(const PageMap& pm, TableWin& tw, int lo_h, int pre, int pre_end,
                                int lo, int hi_all, char* ring, uint64_t* full, int R,
@@ -342,23 +340,27 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
       mbar_init(&wbar[warp], 1);
       if (warp == 0) mbar_init(&fl_bar, 4 * 32);
       fence_mbar_init();
-      hint = read_len(c.seq_len + b);
+      hint = read_len_acquire(c.seq_len + b);
     }
     hint = __shfl_sync(0xffffffffu, hint, 0);
-    if (append && hint < d.max_len) ++hint;  // the length this kernel will attend
+    const bool grows = append && hint < d.max_len;
+    if (grows) ++hint;  // the length this kernel will attend
     __syncwarp();
     const bool hint_flush =
-        append && packed_len(hint, d.residual) > packed_len(hint - 1, d.residual);
+        grows && packed_len(hint, d.residual) > packed_len(hint - 1, d.residual);
     const Plan ph = make_plan(hint, d.residual, NV, hint_flush);
     int lo_h = 0, hi_h = 0, pre = 0, pre_end = 0;
     if (v < ph.np) {
       block_range(ph, v, lo_h, hi_h);
-      // the newest block may be the one the previous kernel is writing
-      pre = tc_pre_issue<BK, BV>(pm, tw, lo_h, hi_h, ph.nb - 1, ring, full, R, pre_end, flag);
+      // The blocks of the published length, but its newest: a decode step
+      // publishes a length while that block may still be on its way to its
+      // page.  The others were written before the length, by kernels that had
+      // ended or (pack.cu) with a fence.
+      const int written = packed_len(grows ? hint - 1 : hint, d.residual) / kGroup - 1;
+      pre = tc_pre_issue<BK, BV>(pm, tw, lo_h, hi_h, written, ring, full, R, pre_end, flag);
       // a decode step that pushes a group out of the window: its owner brings
       // the group's ring rows (old, unchanging) into L2 for the flush
-      if (append && lane == 0 && hi_h == ph.nb && ph.nb > 0 &&
-          ph.Lq > packed_len(hint - 1, d.residual)) {
+      if (hint_flush && lane == 0 && hi_h == ph.nb) {
         prefetch_rows_l2(ring_k, ph.Lq - kGroup, kGroup, d.ring);
         prefetch_rows_l2(ring_v, ph.Lq - kGroup, kGroup, d.ring);
       }
@@ -491,7 +493,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
       seq_ticket == gridDim.y * gridDim.x - 1u) {  // every CTA of b has read L0
     const int L1 = len_s[0];
     __threadfence();
-    c.seq_len[b] = L1;
+    *reinterpret_cast<volatile int*>(c.seq_len + b) = L1;
     reinterpret_cast<unsigned*>(c.seq_len)[d.batch + 2 + b] = 0u;
   }
   if (S == 1) return;

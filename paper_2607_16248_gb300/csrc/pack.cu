@@ -298,9 +298,12 @@ __global__ void __launch_bounds__(kPackThreads)
     __threadfence();
     const unsigned t = atomicAdd(&tickets[b], 1u);
     if (t == (unsigned)d.hkv * gridDim.z - 1u) {
-      c.seq_len[b] = L1;
-      tickets[b] = 0u;
+      // Every CTA's pages and ring rows come before the length (a fence here
+      // as before the tickets): the split plan takes pages by a length that it
+      // reads, with acquire, ahead of its dependency wait.
       __threadfence();
+      *reinterpret_cast<volatile int*>(c.seq_len + b) = L1;
+      tickets[b] = 0u;
     }
   }
 }
