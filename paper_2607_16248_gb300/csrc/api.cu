@@ -543,9 +543,17 @@ kvq_status kvq_drift_metrics(const float* z_fp, const float* z_q, int32_t rows, 
     return fail(KVQ_ERR_ARG, "window must be in [1, k_max] (got %d)", p->window);
   if (!isfinite(p->eps) || !isfinite(p->rho_c))
     return fail(KVQ_ERR_ARG, "eps and rho_c must be finite");
-  trace("kvq_drift_metrics rows %d vocab %d alpha %g window %d k_max %d grid (%d)", rows,
-        vocab, (double)p->alpha, p->window, p->k_max, rows);
-  return cuda_status(launch_drift(z_fp, z_q, rows, vocab, *p, m_t, c_t, d_loc, y_t, cov,
+  DriftPlan plan;
+  const cudaError_t e = drift_plan(rows, vocab, p->alpha, &plan);
+  if (e != cudaSuccess) return cuda_status(e, "kvq_drift_metrics plan");
+  if (plan.stream_threads)
+    trace("kvq_drift_metrics rows %d vocab %d alpha %g window %d k_max %d grid (%d) x %d, then "
+          "(8, %d) x 512 for the rows it leaves", rows, vocab, (double)p->alpha, p->window,
+          p->k_max, rows, plan.stream_threads, plan.clusters);
+  else
+    trace("kvq_drift_metrics rows %d vocab %d alpha %g window %d k_max %d grid (8, %d) x 512",
+          rows, vocab, (double)p->alpha, p->window, p->k_max, plan.clusters);
+  return cuda_status(launch_drift(plan, z_fp, z_q, rows, vocab, *p, m_t, c_t, d_loc, y_t, cov,
                                   static_cast<cudaStream_t>(stream)),
                      "kvq_drift_metrics launch");
 }

@@ -507,9 +507,15 @@ int dgap_max_chunks();
 // Offline drift metrics (drift.cu).
 int drift_max_vocab();
 int drift_max_kcov();
-cudaError_t launch_drift(const float* z_fp, const float* z_q, int rows, int vocab,
-                         const kvq_drift_params& p, int32_t* m_t, float* c_t, float* d_loc,
-                         uint8_t* y_t, float* cov, cudaStream_t st);
+// The kernels of a call: the streaming kernel, one CTA of stream_threads per row
+// (0: none), then the general kernel on `clusters` clusters of eight CTAs.
+struct DriftPlan {
+  int stream_threads, clusters;
+};
+cudaError_t drift_plan(int rows, int vocab, float alpha, DriftPlan* plan);
+cudaError_t launch_drift(const DriftPlan& plan, const float* z_fp, const float* z_q, int rows,
+                         int vocab, const kvq_drift_params& p, int32_t* m_t, float* c_t,
+                         float* d_loc, uint8_t* y_t, float* cov, cudaStream_t st);
 cudaError_t launch_drift_window(const float* cov, int rows, int k_max, float rho_k,
                                 float* mean_cov, int32_t* k_b, cudaStream_t st);
 cudaError_t launch_dgap(const DgapDims& d, const dgap_params& p, float* logits,

@@ -82,7 +82,6 @@ struct Sm {
   u64 xin[kCl][kXw];                // values loaded from the eight CTAs
   u64 xin3[kCl][3 * kXw];           // the same for the three slots of a row's sums
   u64 wsel[kMaxKcov];               // coverage terms of the TopK list
-  float bc[4];                      // broadcast scalars
   uint32_t ru[kW];
   float rf[kW];
 };
@@ -1831,14 +1830,9 @@ cudaError_t launch_stream(const float* z_fp, const float* z_q, int rows, int voc
 }
 }  // namespace
 
-cudaError_t launch_drift(const float* z_fp, const float* z_q, int rows, int vocab,
-                         const kvq_drift_params& p, int32_t* m_t, float* c_t, float* d_loc,
-                         uint8_t* y_t, float* cov, cudaStream_t st) {
+cudaError_t drift_plan(int rows, int vocab, float alpha, DriftPlan* plan) {
   int sms = 0;
-  cudaError_t e = sm_count(&sms);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(drift_general_kernel<false>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Sm));
+  const cudaError_t e = sm_count(&sms);
   if (e != cudaSuccess) return e;
   const int clusters = sms / kCl > 0 ? sms / kCl : 1;
   // A few long rows: a cluster spreads each over eight SMs, and up to 15 run at
@@ -1847,31 +1841,43 @@ cudaError_t launch_drift(const float* z_fp, const float* z_q, int rows, int voca
   // alpha 0.9: 32768: 32 to 36 us streamed, 36 to 40 in clusters; 49152: 36 to 44
   // and 39 to 44; 98304: 51 to 63 and 47 to 54.  alpha 0.99: 24576: 30 to 38 and
   // 36 to 40; 32768: 34 to 44 and 37 to 42; 98304: 56 to 81 and 50 to 59.
-  if (rows * 10 <= sms && vocab > (p.alpha > 0.97f ? 28672 : 40960)) {
-    e = cudaFuncSetAttribute(drift_general_kernel<true>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Sm));
-    if (e != cudaSuccess) return e;
-    drift_general_kernel<true><<<dim3(kCl, rows), kT, sizeof(Sm), st>>>(
-        z_fp, z_q, rows, vocab, p, m_t, c_t, d_loc, y_t, cov);
-    return cudaGetLastError();
+  if (rows * 10 <= sms && vocab > (alpha > 0.97f ? 28672 : 40960)) {
+    plan->stream_threads = 0;
+    plan->clusters = rows;
+  } else {
+    plan->stream_threads = rows <= sms ? 1024 : 512;  // one row per SM: all its threads on it
+    plan->clusters = rows < clusters ? rows : clusters;
   }
-  // at most one row per SM: all of an SM's threads on it
-  e = rows <= sms ? launch_stream<1024>(z_fp, z_q, rows, vocab, p, m_t, c_t, d_loc, y_t, cov, st)
-                  : launch_stream<512>(z_fp, z_q, rows, vocab, p, m_t, c_t, d_loc, y_t, cov, st);
+  return cudaSuccess;
+}
+
+cudaError_t launch_drift(const DriftPlan& plan, const float* z_fp, const float* z_q, int rows,
+                         int vocab, const kvq_drift_params& p, int32_t* m_t, float* c_t,
+                         float* d_loc, uint8_t* y_t, float* cov, cudaStream_t st) {
+  const auto general =
+      plan.stream_threads ? drift_general_kernel<false> : drift_general_kernel<true>;
+  cudaError_t e = cudaFuncSetAttribute(general, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)sizeof(Sm));
   if (e != cudaSuccess) return e;
-  // the rows it leaves: usually none, so the launch overlaps its end
+  if (plan.stream_threads) {
+    e = plan.stream_threads == 1024
+            ? launch_stream<1024>(z_fp, z_q, rows, vocab, p, m_t, c_t, d_loc, y_t, cov, st)
+            : launch_stream<512>(z_fp, z_q, rows, vocab, p, m_t, c_t, d_loc, y_t, cov, st);
+    if (e != cudaSuccess) return e;
+  }
+  // behind a streaming kernel: the rows it leaves, usually none, so the launch
+  // overlaps its end
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  cfg.gridDim = dim3(kCl, rows < clusters ? rows : clusters);
+  cfg.numAttrs = plan.stream_threads ? 1 : 0;
+  cfg.gridDim = dim3(kCl, plan.clusters);
   cfg.blockDim = dim3(kT);
   cfg.dynamicSmemBytes = sizeof(Sm);
   cfg.stream = st;
-  return cudaLaunchKernelEx(&cfg, drift_general_kernel<false>, z_fp, z_q, rows, vocab, p, m_t,
-                            c_t, d_loc, y_t, cov);
+  return cudaLaunchKernelEx(&cfg, general, z_fp, z_q, rows, vocab, p, m_t, c_t, d_loc, y_t, cov);
 }
 
 cudaError_t launch_drift_window(const float* cov, int rows, int k_max, float rho_k,
