@@ -1396,7 +1396,11 @@ __global__ void __launch_bounds__(kS, 1024 / kS)
   // mass outside C.  z_q below cut_q, the least of the warps' maxima of 256
   // elements (the upper 1.2% or 1.5% of the row in the middle), is not a
   // candidate when k_max is under 1/400 of the vocabulary.
+  // Two kinds of row are seen here to be the general kernel's: with alpha = 1 a
+  // token that still has mass below the grid, and logits so close together
+  // that their bins hold far more than the lists do.
   float mf = -INFINITY, mq = -INFINITY, cut_f, cut_q;
+  float least = INFINITY, least_mass = INFINITY;  // of all and of those with mass
   {
     float z[kRuns];
 #pragma unroll
@@ -1416,14 +1420,24 @@ __global__ void __launch_bounds__(kS, 1024 / kS)
     // (a warp's terms are relative to its own maximum)
     float e = 0.0f;
 #pragma unroll
-    for (int u = 0; u < kRuns; ++u)
+    for (int u = 0; u < kRuns; ++u) {
       e += z[u] > -INFINITY ? exp2f((z[u] - mf) * 1.44269504f) : 0.0f;
+      const int i = n >= kRuns * kS ? u * (n / kRuns) + t : u * kS + t;
+      least = fminf(least, i < n ? z[u] : INFINITY);
+      least_mass = fminf(least_mass, z[u] > mf - 27.0f ? z[u] : INFINITY);
+    }
 #pragma unroll
-    for (int o = 16; o; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+    for (int o = 16; o; o >>= 1) {
+      e += __shfl_xor_sync(0xffffffffu, e, o);
+      least = fminf(least, __shfl_xor_sync(0xffffffffu, least, o));
+      least_mass = fminf(least_mass, __shfl_xor_sync(0xffffffffu, least_mass, o));
+    }
     if (lane == 0) {
       s.rf[0][warp] = mf;
       s.rf[1][warp] = mq;
       s.rf[2][warp] = e;
+      s.rf[3][warp] = least;
+      s.su[warp] = __float_as_uint(least_mass);
     }
     __syncthreads();
     // second level: lane = warp
@@ -1432,8 +1446,12 @@ __global__ void __launch_bounds__(kS, 1024 / kS)
     cut_q = lane < kSw ? qw : INFINITY;
     mf = mw;
     mq = qw;
+    least = lane < kSw ? s.rf[3][lane] : INFINITY;
+    least_mass = lane < kSw ? __uint_as_float((uint32_t)s.su[lane]) : INFINITY;
 #pragma unroll
     for (int o = 16; o; o >>= 1) {
+      least = fminf(least, __shfl_xor_sync(0xffffffffu, least, o));
+      least_mass = fminf(least_mass, __shfl_xor_sync(0xffffffffu, least_mass, o));
       mf = fmaxf(mf, __shfl_xor_sync(0xffffffffu, mf, o));
       mq = fmaxf(mq, __shfl_xor_sync(0xffffffffu, mq, o));
       cut_q = fminf(cut_q, __shfl_xor_sync(0xffffffffu, cut_q, o));
@@ -1451,6 +1469,11 @@ __global__ void __launch_bounds__(kS, 1024 / kS)
   }
   const float af = (float)bin_origin(mf), aq = (float)bin_origin(mq);
   const float m0 = mf > -INFINITY ? mf : 0.0f;  // reference of the guess
+  if ((p.alpha >= 1.0f && least_mass < bin_floor(af)) ||
+      (mf - least) * kDepthScale + 1.0f < (float)(n / (4 * kL))) {
+    if (t == 0) m_t[row] = -1;
+    return;
+  }
 
   // ---- pass A (z_fp last: pass B reads it again) ----
   int n_cand = 0;  // z_q candidates of this thread
@@ -1804,17 +1827,33 @@ int drift_max_kcov() { return kMaxKcov; }
 int drift_cap() { return kCap; }
 
 namespace {
-// SMs of the current device (looked up once per device).
-cudaError_t sm_count(int* sms) {
-  static std::atomic<int> known[64];
+// SMs of the current device and the clusters of the general kernel that it runs
+// at once (looked up once per device; 152 SMs do not hold 19 of them: a second
+// wave of the rest took 1.6 times as long).
+cudaError_t device_limits(int* sms, int* clusters) {
+  static std::atomic<int> known[64];  // clusters << 16 | SMs
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  *sms = dev < 64 ? known[dev].load(std::memory_order_relaxed) : 0;
-  if (*sms > 0) return cudaSuccess;
-  e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess && dev < 64) known[dev].store(*sms, std::memory_order_relaxed);
-  return e;
+  int k = dev < 64 ? known[dev].load(std::memory_order_relaxed) : 0;
+  if (k == 0) {
+    e = cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(drift_general_kernel<false>,
+                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Sm));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kCl, *sms);
+    cfg.blockDim = dim3(kT);
+    cfg.dynamicSmemBytes = sizeof(Sm);
+    if (e == cudaSuccess)
+      e = cudaOccupancyMaxActiveClusters(clusters, drift_general_kernel<false>, &cfg);
+    if (e != cudaSuccess) return e;
+    k = (*clusters < 1 ? 1 : *clusters) << 16 | *sms;
+    if (dev < 64) known[dev].store(k, std::memory_order_relaxed);
+  }
+  *sms = k & 0xffff;
+  *clusters = k >> 16;
+  return cudaSuccess;
 }
 
 template <int kS>
@@ -1831,17 +1870,20 @@ cudaError_t launch_stream(const float* z_fp, const float* z_q, int rows, int voc
 }  // namespace
 
 cudaError_t drift_plan(int rows, int vocab, float alpha, DriftPlan* plan) {
-  int sms = 0;
-  const cudaError_t e = sm_count(&sms);
+  int sms = 0, clusters = 0;
+  const cudaError_t e = device_limits(&sms, &clusters);
   if (e != cudaSuccess) return e;
-  const int clusters = sms / kCl > 0 ? sms / kCl : 1;
   // A few long rows: a cluster spreads each over eight SMs, and up to 15 run at
   // once.  The line lies where a CTA's stream of a row takes as long, which
   // falls with alpha (more of the row belongs to C): 7 rows, sigma 2.1 to 3.9,
   // alpha 0.9: 32768: 32 to 36 us streamed, 36 to 40 in clusters; 49152: 36 to 44
   // and 39 to 44; 98304: 51 to 63 and 47 to 54.  alpha 0.99: 24576: 30 to 38 and
   // 36 to 40; 32768: 34 to 44 and 37 to 42; 98304: 56 to 81 and 50 to 59.
-  if (rows * 10 <= sms && vocab > (alpha > 0.97f ? 28672 : 40960)) {
+  // With alpha = 1 every token with mass belongs to C, and a streamed row takes
+  // as long as three waves of clusters where it is settled at all: 16 rows of
+  // 128256, sigma 1 and 3: 196 and 116 us streamed, 112 in clusters.
+  if ((rows * 10 <= sms && vocab > (alpha > 0.97f ? 28672 : 40960)) ||
+      (alpha >= 1.0f && rows * 10 <= 3 * sms)) {
     plan->stream_threads = 0;
     plan->clusters = rows;
   } else {
