@@ -644,7 +644,7 @@ def run_gpu(args, spec):
            "layers": s["layers"], "vocab": s["vocab"], "residual": 128, "group": 32,
            "dgap_K": DGAP_K, "dgap_hidden": DGAP_HIDDEN, "tau": round(st.dgap.tau, 6),
            "n_splits": st.n_splits,
-           "plan": ("flat: every pair's blocks and window chunks cut into equal per-warp "
+           "plan": ("flat: every pair's blocks and window units cut into equal per-warp "
                     "ranges over one CTA per SM" if st.n_splits == 0 else
                     f"split: {st.n_splits} CTAs per (sequence, kv-head)"),
            "kv_layout": (f"paged: block table over a shuffled pool of {st.paged_pages} page sets "

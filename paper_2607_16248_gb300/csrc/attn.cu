@@ -500,6 +500,7 @@ __device__ __forceinline__ void prefetch_rows_l2(const __half* ring_base, int p0
 // L1, so that a later read sees the table as it is then).
 __device__ __forceinline__ void prefetch_pages_l2(const PageMap& pm, int j0, int j1) {
   const int lane = threadIdx.x & 31;
+  if (j1 <= j0) return;
   for (int j = j0 + lane; j < (pm.paged() ? j1 : j0 + 1); j += 32) {
     const char* src = pm.at(j, pm.paged() ? __ldcg(pm.row + j) : 0);
     const uint32_t bytes = (uint32_t)((pm.paged() ? 1 : j1 - j0) * pm.page);
@@ -511,9 +512,9 @@ __device__ __forceinline__ void prefetch_pages_l2(const PageMap& pm, int j0, int
 // Window units [i0, i1) of one pair (unit u = tokens Lq + 16 u ...), K and V
 // rows staged together in the warp's (idle) ring; *phase_io is the parity
 // count of the warp's staging barrier, kept across calls.  A bounded wait that
-// gives up sets KVQ_FLAG_WAIT_TIMEOUT and ends them.  (32-token chunks, whose
-// V rows waited for the K rows' place, made one item of two round trips: in a
-// launch with little work the warps that held one ended last.)
+// gives up sets KVQ_FLAG_WAIT_TIMEOUT and ends them.  (32-token units, whose V
+// rows wait for the K rows' place, are items of two round trips, and in a launch
+// with little work the warps that hold one end last.)
 // Out of line, like tc_packed_warp.
 template <int BK, int BV, bool kWide>
 __device__ __noinline__ TcState tc_window_units(TcState st, const Dims d, const __half* ring_k,

@@ -179,18 +179,16 @@ __device__ __forceinline__ RowSrc make_src(const Dims& d, const kvq_cache& c, co
 // ring), so no staging tile and no shared-memory atomics; many small CTAs
 // keep the loads of many blocks in flight.  The ring keeps its rows until the
 // append kernel behind this one.  grid (blocks, hkv, batch_count) of 128
-// threads.  (With the four or five blocks that begin in the ring left to the
-// append kernel, one after another in one CTA per kv-head, a 4099-token chunk
-// of 4 x 8 heads at 4 bits took 49 us; here they are CTAs like the others.
-// Only their loads differ: an out-of-line call for them cost the kernel 7 to 11
-// registers.)
+// threads.  Blocks that begin in the ring differ in their loads only (4099
+// tokens of 4 x 8 heads at 4 bits: 26 us a chunk, 49 with those blocks one
+// after another in the append kernel).
 constexpr int kInputThreads = 4 * 32;
 
 // Nine CTAs per SM (56 registers) and eight for K8V8 (64): more loads in flight
 // where two code bodies also miss in the instruction cache.  128k tokens of 8
-// heads, K4V2 with 6, 7, 8 and 9 CTAs: 221, 206, 191 and 180 us (201 at first),
-// K8V4 235, 217, 204 and 196; K4V4 147 with 8, 140 with 9; K8V8 188 with 8, 198
-// with 9, and ten spill in the equal widths (K4V4 154).
+// heads, K4V2 with 6, 7, 8 and 9 CTAs: 221, 206, 191 and 180 us, K8V4 235, 217,
+// 204 and 196; K4V4 147 with 8, 140 with 9; K8V8 188 with 8, 198 with 9, and ten
+// spill in the equal widths (K4V4 154).
 template <int BK, int BV>
 __global__ void __launch_bounds__(kInputThreads, BK == 8 && BV == 8 ? 8 : 9)
     pack_input_blocks_kernel(Dims d, kvq_cache c, const __half* __restrict__ k_new,
